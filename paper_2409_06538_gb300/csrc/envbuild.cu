@@ -142,9 +142,9 @@ template <typename T, int CHI> struct JStride {
 
 template <typename T, int CHI>
 __host__ __device__ constexpr size_t env_smem_elems() {
-  // CHI = 64: only Y and V (D*DP each) and the Householder vectors (three of 2D) stay in shared memory;
+  // CHI = 64: only Y and V (D*DP each) and the reflector slots (16 of 2D) stay in shared memory;
   // M lives in per-realization global scratch and R, the tile are read from global memory
-  if (CHI > 32) return (size_t)2 * (2 * CHI) * JStride<T, CHI>::DP + (size_t)6 * (2 * CHI);
+  if (CHI > 32) return (size_t)2 * (2 * CHI) * JStride<T, CHI>::DP + (size_t)32 * (2 * CHI);
   // backward: M, R (D*D each), Y, V (D*DP each) + tile (2*CHI*CHI); P (D*CHI) lives in the Y
   //           region and Q (2*CHI*CHI) in the V region between their uses
   // forward : X (2D*D, aliases M and Y) + R (D*D) + tile; the Householder vectors use V
@@ -153,140 +153,222 @@ __host__ __device__ constexpr size_t env_smem_elems() {
          (size_t)2 * CHI * CHI;
 }
 
-// Householder R factor of the first nc <= NC columns of an MR-row matrix A (column j at
-// A + j*ld) in place, by all threads of the CTA: warp j % NWARP owns column j; reflector j is
-// applied to every column a warp owns with the dot products reduced in one interleaved
-// butterfly, and the owner of column j+1 forms reflector j+1 first, deferring its other columns
-// by one step (reflectors rotate through three slots of vbuf).  On return the upper triangle of
-// A holds R, zeros below.  With vsave (MR x NC, column j = reflector j, zero above row j) and
-// csave (nc coefficients 2/|v|^2) the reflectors are kept, so that Q = H_0 H_1 ... H_{nc-1} can
-// be applied afterwards.  Not inlined: one body serves both QRs of a site (measured 3 % faster
-// than two inlined copies).  A Givens QR in the parallel Sameh-Kuck order (one barrier per
-// stage, no reductions) measured slower per QR and less accurate once Q is accumulated.
-template <typename T, int MR, int NC, int NWARP>
-__device__ __noinline__ void householder_r(T* A, int ld, int nc, T (*vbuf)[MR], T* vcoef, T* vsave,
-                                              T* csave, int lane, int warp) {
-  constexpr int RPL = MR / 32 > 0 ? MR / 32 : 1;
-  constexpr int CPW = (NC + NWARP - 1) / NWARP;
+// Householder QR with the matrix in registers.  A group of G lanes owns CPT columns of the MR x NC
+// matrix, lane g of a group the rows g + G u (u < RPT); warp w owns the CW consecutive columns from
+// w CW on.  Reflector j is formed by the group that owns column j, published in shared memory, and
+// applied by every group to its later columns.
+//
+// Every sum over the rows has one fixed association, whatever G: 32 partial sums, partial l over the
+// rows l, l + 32, ... in this order, then the butterfly l ^ 16, 8, 4, 2, 1.  A lane holds the partials
+// l = g mod G, so the levels down to G are register adds and only log2(G) shuffles remain.
+//
+// What bounds it: the chain dot product -> shuffles -> update -> norm -> square root -> publish of
+// consecutive pivots (about 700 cycles each at 64 x 64, 520 in one warp), not the arithmetic.  With the
+// columns in shared memory a reflector cost 1440 cycles: every step read and wrote the whole matrix
+// there and reduced each dot product over 32 lanes, 870 cycles of the shared-memory pipe alone.
+// 16 rows a lane and log2(MR/16) shuffle levels balance the serial adds of a lane against the
+// shuffles (30 cycles a level).  Environment build at chi = 32, FP32 (one GB300): 203 -> 150 us a site
+// step with one realization per SM (L = 64), 331 -> 214 us with three (L = 48).
+template <typename T, int MR, int NC> struct QrCfg {
+  static constexpr int G = MR >= 32 ? MR / 16 : 2;          // lanes of a column: 16 rows each from MR = 32 on
+  static constexpr int RPT = MR / G;
+  static constexpr int NVL = 32 / G < RPT ? 32 / G : RPT;   // partial sums a lane holds
+  static constexpr int NRUN = RPT / 4;                      // runs of four rows a lane holds
+  static constexpr int CPT = NC * G > 512 ? (NC * G) / 512 : (NC * G > 256 ? 2 : 1);
+  static constexpr int NTQ = NC * G / CPT < 32 ? 32 : NC * G / CPT;   // threads taking part
+  static constexpr int GPW = 32 / G;                        // groups of a warp
+  static constexpr int CW = GPW * CPT;                      // columns of a warp
+  static constexpr int RING = NTQ == 32 ? 2 : 16;           // reflector slots in turn
+};
+// Place of row i in a column stored for QrCfg: each lane's rows in 16-byte runs of four, the runs of
+// the G lanes side by side, so that a group reads its column in conflict-free vector loads.
+template <int G> __device__ __forceinline__ int qr_pos(int i) {
+  const int g = i % G, u = i / G;
+  return (u >> 2) * (4 * G) + g * 4 + (u & 3);
+}
+
+// Two FP32 operations in one instruction (fma.rn.f32x2, add.rn.f32x2): the same roundings, half the
+// issue slots.
+__device__ __forceinline__ unsigned long long pack2(float a, float b) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpack2(unsigned long long r, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(r));
+}
+// c += a * b, p += q on pairs of adjacent array elements
+__device__ __forceinline__ void fma_pair(const float* a, const float* b, float* c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(pack2(a[0], a[1])), "l"(pack2(b[0], b[1])), "l"(pack2(c[0], c[1])));
+  unpack2(r, c[0], c[1]);
+}
+__device__ __forceinline__ void add_pair(float* p, const float* q) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(p[0], p[1])), "l"(pack2(q[0], q[1])));
+  unpack2(r, p[0], p[1]);
+}
+__device__ __forceinline__ void fma_pair(const double* a, const double* b, double* c) {
+  c[0] = fma(a[0], b[0], c[0]);
+  c[1] = fma(a[1], b[1], c[1]);
+}
+__device__ __forceinline__ void add_pair(double* p, const double* q) { p[0] += q[0]; p[1] += q[1]; }
+
+// Sum of v * x over the rows of the runs C0 and later (the earlier ones hold zeros) in the fixed
+// association; every lane of the group gets it.
+template <typename Q, int C0, typename T>
+__device__ __forceinline__ T qr_dot(const T (&v)[Q::RPT], const T (&x)[Q::RPT]) {
+  T p[Q::NVL];
+#pragma unroll
+  for (int a = 0; a < Q::NVL; ++a) p[a] = T(0);
+#pragma unroll
+  for (int u = 4 * C0; u < Q::RPT; u += 2) fma_pair(v + u, x + u, p + u % Q::NVL);
+#pragma unroll
+  for (int lv = Q::NVL / 2; lv > 1; lv >>= 1)
+#pragma unroll
+    for (int a = 0; a < lv; a += 2) add_pair(p + a, p + a + lv);
+  T d = p[0] + p[1];
+#pragma unroll
+  for (int o = Q::G / 2; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+  return d;
+}
+template <typename Q, int C0, typename T>
+__device__ __forceinline__ void qr_update(T md, const T (&v)[Q::RPT], T (&x)[Q::RPT]) {
+  const T m2[2] = {md, md};
+#pragma unroll
+  for (int u = 4 * C0; u < Q::RPT; u += 2) fma_pair(m2, v + u, x + u);
+}
+template <typename Q, int C0, typename T>
+__device__ __forceinline__ void qr_load_v(const T* vs, int g, T (&v)[Q::RPT]) {
+#pragma unroll
+  for (int ch = C0; ch < Q::NRUN; ++ch) ld4(vs + ch * 4 * Q::G + g * 4, v + 4 * ch);
+}
+__device__ __forceinline__ void named_arrive(int id, int nthreads) {
+  asm volatile("bar.arrive %0, %1;\n" ::"r"(id), "r"(nthreads) : "memory");
+}
+
+// State of one factorisation: where the reflectors go and how they are handed on.
+// The warp that owns the pivot columns runs ahead: it publishes reflector after reflector with
+// bar.arrive and only the others wait.  The published reflectors use eight barriers in turn, and
+// with every eighth the pivot's warp waits too, so that no barrier is used again before all have
+// passed it; the reflector slots (16 in turn unless all are kept) follow from the same count: a slot is
+// written again only after a barrier that all have passed since they read it.
+template <typename T> struct QrOut {
+  T* vring;          // slots of MR elements
+  bool keep_all;     // slot j holds reflector j, else published reflector k is in slot k mod RING
+  T* vsave;          // the reflectors once more, at j * MR (nullable)
+  T* cden;           // [j]: reflector j's coefficient 2/|v|^2 (0: no reflector), with kLate its reciprocal
+  T* diag;           // [j]: R_jj
+};
+// In FP32 every warp inverts the coefficient beside its dot products, off the pivots' chain; in FP64,
+// where a division occupies the FP64 pipe, only the pivot's warp does.
+template <typename T> constexpr bool kLate = sizeof(T) == 4;
+
+// Reflector of column j, by the warp that owns it; j lies in the rows of run C0.
+template <typename T, int MR, int NC, int C0>
+__device__ __forceinline__ void qr_pivot(T (&x)[QrCfg<T, MR, NC>::CPT][QrCfg<T, MR, NC>::RPT], int j, T* vs,
+                                         const QrOut<T>& o, int g, int gi, int warp) {
+  using Q = QrCfg<T, MR, NC>;
+  constexpr int G = Q::G;
   const T tiny = (sizeof(T) == 4) ? T(1e-36) : T(1e-300);
-  auto house = [&](int j) {
-    T* col = A + (size_t)j * ld;
-    T xr[RPL];
-    T ss = 0;
+  const int jl = j - warp * Q::CW, jq = jl / Q::GPW, jr = j - 4 * G * C0;   // row of the pivot within the run
 #pragma unroll
-    for (int t = 0; t < RPL; ++t) {
-      const int i = lane + 32 * t;
-      xr[t] = (i < MR && i >= j) ? col[i] : T(0);
-      ss += xr[t] * xr[t];
+  for (int q = 0; q < Q::CPT; ++q) {
+    if (Q::CPT > 1 && q != jq) continue;     // warp-uniform
+    T xr[Q::RPT], x0 = T(0);
+#pragma unroll
+    for (int u = 4 * C0; u < Q::RPT; ++u) xr[u] = x[q][u];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int i = g + G * u;               // rows above the pivot belong to R
+      if (i < jr) xr[4 * C0 + u] = T(0);
+      if (i == jr) x0 = xr[4 * C0 + u];
     }
-    ss = warp_sum(ss);
-    const T x0 = col[j];
-    __syncwarp();
-    T* vj = vbuf[j % 3];
-    T coef = T(0);
-    if (ss <= tiny) {
-#pragma unroll
-      for (int t = 0; t < RPL; ++t) {
-        const int i = lane + 32 * t;
-        if (i < MR) { vj[i] = T(0); if (i > j) col[i] = T(0); if (vsave) vsave[(size_t)j * MR + i] = T(0); }
-      }
-    } else {
-      const T nrm = num<T>::sqrt_(ss);
+    const T ss = qr_dot<Q, C0, T>(xr, xr);
+    const bool null = ss <= tiny;
+    const T nrm = num<T>::sqrt_(ss);
+    if (gi == jl - jq * Q::GPW) {            // the pivot's group
       const T alpha = x0 >= T(0) ? -nrm : nrm;
       const T v0 = x0 - alpha;
 #pragma unroll
-      for (int t = 0; t < RPL; ++t) {
-        const int i = lane + 32 * t;
-        if (i < MR) {
-          const T vi = (i == j) ? v0 : xr[t];
-          vj[i] = vi;
-          if (vsave) vsave[(size_t)j * MR + i] = vi;
-          if (i >= j) col[i] = (i == j) ? alpha : T(0);
-        }
+      for (int u = 0; u < 4; ++u)
+        if (g + G * u == jr) { xr[4 * C0 + u] = v0; if (!null) x[q][4 * C0 + u] = alpha; }
+#pragma unroll
+      for (int ch = C0; ch < Q::NRUN; ++ch) {
+        st4(vs + ch * 4 * G + g * 4, xr + 4 * ch);
+        if (o.vsave) st4(o.vsave + (size_t)j * MR + ch * 4 * G + g * 4, xr + 4 * ch);
       }
-      coef = T(1) / (nrm * (nrm + (x0 >= T(0) ? x0 : -x0)));
-    }
-    if (lane == 0) { vcoef[j % 3] = coef; if (csave) csave[j] = coef; }
-  };
-  auto apply1 = [&](int jj, int k) {
-    const T coef = vcoef[jj % 3];
-    if (coef == T(0)) return;
-    const T* v = vbuf[jj % 3];
-    T* col = A + (size_t)k * ld;
-    T xr[RPL], vr[RPL];
-    T d = 0;
-#pragma unroll
-    for (int t = 0; t < RPL; ++t) {
-      const int i = lane + 32 * t;
-      xr[t] = i < MR ? col[i] : T(0);
-      vr[t] = i < MR ? v[i] : T(0);
-      d += vr[t] * xr[t];
-    }
-    d = warp_sum(d) * coef;
-#pragma unroll
-    for (int t = 0; t < RPL; ++t) { const int i = lane + 32 * t; if (i < MR) col[i] = xr[t] - d * vr[t]; }
-  };
-  auto apply_batch = [&](int jj, int lo) {
-    const T coef = vcoef[jj % 3];
-    if (coef == T(0)) return;
-    const T* v = vbuf[jj % 3];
-    T vr[RPL], d[CPW];
-#pragma unroll
-    for (int t = 0; t < RPL; ++t) { const int i = lane + 32 * t; vr[t] = i < MR ? v[i] : T(0); }
-#pragma unroll
-    for (int q = 0; q < CPW; ++q) {
-      const int k = warp + NWARP * q;
-      d[q] = 0;
-      if (k > lo && k < nc) {
-        const T* col = A + (size_t)k * ld;
-#pragma unroll
-        for (int t = 0; t < RPL; ++t) { const int i = lane + 32 * t; if (i < MR) d[q] += vr[t] * col[i]; }
+      if (g == jr % G) {
+        const T den = nrm * (nrm + (x0 >= T(0) ? x0 : -x0));
+        o.cden[j] = null ? T(0) : (kLate<T> ? den : T(1) / den);
+        o.diag[j] = null ? x0 : alpha;
       }
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-      for (int q = 0; q < CPW; ++q) d[q] += __shfl_xor_sync(0xffffffffu, d[q], o);
-#pragma unroll
-    for (int q = 0; q < CPW; ++q) {
-      const int k = warp + NWARP * q;
-      if (k > lo && k < nc) {
-        T* col = A + (size_t)k * ld;
-        const T dc = d[q] * coef;
-#pragma unroll
-        for (int t = 0; t < RPL; ++t) { const int i = lane + 32 * t; if (i < MR) col[i] -= dc * vr[t]; }
-      }
-    }
-  };
-  __syncthreads();
-  if (nc <= 0) return;
-  if (warp == 0) house(0);
-  int pend = -1;
-  for (int j = 0; j < nc; ++j) {
-    __syncthreads();
-    if (pend >= 0) { apply_batch(pend, pend + 1); pend = -1; }
-    const int nxt = j + 1;
-    if (nxt < nc && warp == nxt % NWARP) {
-      apply1(j, nxt);
-      __syncwarp();
-      house(nxt);
-      pend = j;
-    } else {
-      apply_batch(j, j);
-    }
-    __syncwarp();
   }
-  __syncthreads();
 }
 
-template <int CHI> struct Pair {
-  // round-robin ("circle") schedule over n columns (n even): n-1 rounds of n/2 disjoint pairs
-  static __device__ __forceinline__ void get(int n, int round, int w, int& p, int& q) {
-    const int m = n - 1;
-    if (w == 0) { p = n - 1; q = round; }
-    else { p = (round + w) % m; q = (round - w + m) % m; }
+// The pivots whose rows lie in run C0, then those of the later runs.
+template <typename T, int MR, int NC, int C0, typename Skip>
+__device__ __forceinline__ void qr_runs(T (&x)[QrCfg<T, MR, NC>::CPT][QrCfg<T, MR, NC>::RPT], int nc, int& pub,
+                                        const QrOut<T>& o, int g, int gi, int warp, Skip skip) {
+  using Q = QrCfg<T, MR, NC>;
+  constexpr int J0 = 4 * Q::G * C0, J1 = J0 + 4 * Q::G < NC ? J0 + 4 * Q::G : NC;
+  auto slot = [&](int j) { return o.vring + (size_t)(o.keep_all ? j : pub % Q::RING) * MR; };
+  const int first = warp * Q::CW, last = first + Q::CW - 1;
+  const int je = nc < J1 ? nc : J1;
+  if (J0 < je && J0 >= first && J0 <= last && !skip(J0)) qr_pivot<T, MR, NC, C0>(x, J0, slot(J0), o, g, gi, warp);
+  for (int j = J0; j < je; ++j) {
+    const bool live = !skip(j);
+    if (live) {
+      if constexpr (Q::NTQ == 32) __syncwarp();
+      else if (j >= first && j <= last && (pub & 7) != 7) { __syncwarp(); named_arrive(2 + (pub & 7), Q::NTQ); }
+      else named_barrier(2 + (pub & 7), Q::NTQ);
+      if (last > j) {
+        T v[Q::RPT];
+        qr_load_v<Q, C0, T>(slot(j), g, v);
+        const T den = o.cden[j];
+        const T coef = !kLate<T> || den == T(0) ? den : T(1) / den;
+#pragma unroll
+        for (int q = 0; q < Q::CPT; ++q) {
+          T d = qr_dot<Q, C0, T>(v, x[q]) * coef;
+          if (first + q * Q::GPW + gi <= j) d = T(0);
+          qr_update<Q, C0>(-d, v, x[q]);
+        }
+      }
+      ++pub;
+    }
+    const int nx = j + 1;
+    if (nx < je && nx >= first && nx <= last && !skip(nx)) qr_pivot<T, MR, NC, C0>(x, nx, slot(nx), o, g, gi, warp);
   }
-};
+  if constexpr (J1 < NC) qr_runs<T, MR, NC, C0 + 1>(x, nc, pub, o, g, gi, warp, skip);
+}
+
+// Factor the columns j < nc for which skip(j) is false (skip(j): the column is known to be zero, so
+// its reflector is the identity; it must be the same for every thread).  On return x holds R on and
+// above the diagonal (below it, what is left of the reflectors).
+template <typename T, int MR, int NC, typename Skip>
+__device__ __forceinline__ void qr_factor(T (&x)[QrCfg<T, MR, NC>::CPT][QrCfg<T, MR, NC>::RPT], int nc,
+                                          const QrOut<T>& o, int lane, int warp, Skip skip) {
+  using Q = QrCfg<T, MR, NC>;
+  int pub = 0;                              // reflectors published
+  qr_runs<T, MR, NC, 0>(x, nc, pub, o, lane % Q::G, lane / Q::G, warp, skip);
+}
+
+// x <- H_0 H_1 ... H_{n-1} x for one column per group, the reflectors as qr_factor kept them.
+template <typename T, int MR, int NC, int C0 = (NC - 1) / (4 * QrCfg<T, MR, NC>::G)>
+__device__ __forceinline__ void qr_apply_q(T (&x)[QrCfg<T, MR, NC>::RPT], int n, const T* vs, const T* coefs, int g) {
+  using Q = QrCfg<T, MR, NC>;
+  constexpr int J0 = 4 * Q::G * C0, J1 = J0 + 4 * Q::G < NC ? J0 + 4 * Q::G : NC;
+  for (int j = (n < J1 ? n : J1) - 1; j >= J0; --j) {
+    const T coef = coefs[j];
+    if (coef == T(0)) continue;
+    T v[Q::RPT];
+    qr_load_v<Q, C0, T>(vs + (size_t)j * MR, g, v);
+    const T d = qr_dot<Q, C0, T>(v, x) * coef;
+    qr_update<Q, C0>(-d, v, x);
+  }
+  if constexpr (C0 > 0) qr_apply_q<T, MR, NC, C0 - 1>(x, n, vs, coefs, g);
+}
 
 template <typename T, typename TE, int CHI>
 __global__ void __launch_bounds__(EnvCfg<CHI>::NT, (sizeof(T) == 8 || CHI > 32) ? 1 : 3)
@@ -321,14 +403,15 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
   T* Xs = sm;                 // 2D x D col-major
 
   __shared__ T Wc[8];               // W[x][a][b] at x*4 + a*2 + b
-  int8_t* jv_s = reinterpret_cast<int8_t*>(kBig ? Vc + D * DP + 6 * D : Bt + TILE);   // Jv[r][c], L entries
+  int8_t* jv_s = reinterpret_cast<int8_t*>(kBig ? Vc + D * DP + 32 * D : Bt + TILE);   // Jv[r][c], L entries
   int8_t* jh_s = jv_s + args.L;                                // Jh[r+1][c], L-1 entries
   const T eb = (T)exp(beta), ebm = (T)exp(-beta);             // exp(+-beta): every Boltzmann weight
-  // Householder vectors (three slots; the V region is idle in the forward sweep unless
-  // the forward matrix X fills Y and V, as for kBig)
-  T (*vbuf)[2 * D] = reinterpret_cast<T (*)[2 * D]>(kBig ? Vc + D * DP : Vc);
-  __shared__ T vcoef[3];
-  __shared__ T csave[D];            // coefficients of the backward sweep's second QR
+  using QF = QrCfg<T, 2 * D, D>;     // the forward sweep's QR
+  using QB = QrCfg<T, D, D>;         // the backward sweep's
+  // reflector slots (the V region is idle in the forward sweep unless X fills Y and V, as for kBig)
+  T* const vfwd = kBig ? Vc + D * DP : Vc;
+  __shared__ T csave[D];            // the reflectors' coefficients (as qr_factor leaves them, then inverted)
+  __shared__ T diag[D];
   __shared__ T red[32];
   __shared__ T sig[D];
   __shared__ int sel[CHI];
@@ -408,9 +491,8 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
     // R_0 = [1]
     if constexpr (kBig) Rc = Rstore;
     for (int e = tid; e < D * D; e += NT) Rc[e] = (e == 0) ? T(1) : T(0);
-    if (!kBig && tid == 0) {
-      for (int e = 0; e < D * D; ++e) Rstore[e] = (e == 0) ? T(1) : T(0);
-    }
+    if constexpr (!kBig)
+      for (int e = tid; e < D * D; e += NT) Rstore[e] = (e == 0) ? T(1) : T(0);
     // the tile the first sweep starts on: site 0 (forward sweep), frame site L-1 (zip-up)
     if constexpr (!kBig) prefetch_async(Bt, prev + (size_t)(zip ? osite(L - 1) : 0) * TILE, TILE * (int)sizeof(T), tid, NT);
     __syncthreads();
@@ -453,147 +535,47 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
         for (int jj = 0; jj < 4; ++jj) {
           T* xc = Xs + (size_t)(b * CHI + b0 + jj) * (2 * D);
 #pragma unroll
-          for (int ii = 0; ii < 4; ++ii) xc[2 * (i0 + ii) + x] = acc[ii][jj];
+          for (int ii = 0; ii < 4; ++ii) xc[qr_pos<QF::G>(2 * (i0 + ii) + x)] = acc[ii][jj];
         }
       }
       __syncthreads();
       // the next site's tile streams in while the QR runs
       if constexpr (!kBig) prefetch_async(Bt, prev + (size_t)(c + 1) * TILE, TILE * (int)sizeof(T), tid, NT);
-      // Householder QR of X (m = 2D rows, D columns); warp (j % NWARP) owns column j.
-      constexpr int m = 2 * D;
-      const T tiny = (sizeof(T) == 4) ? T(1e-36) : T(1e-300);
-      // Each lane owns rows lane + 32 t (t < m/32) of a column; the reflector vector is
-      // stored zero above its pivot row, so the updates run over all rows unconditionally.
-      constexpr int RPL = m / 32 > 0 ? m / 32 : 1;     // rows per lane
-      constexpr int CPW = (D + NWARP - 1) / NWARP;      // columns a warp owns: k = warp + NWARP t
-      auto house = [&](int j) {   // executed by the owning warp for column j
-        T* col = Xs + (size_t)j * m;
-        T xr[RPL];
-        T ss = 0;
+      // R factor of X in registers; R_{c+1} = R / max |R_jj| (col-major, zeros below the diagonal)
+      if (warp < QF::NTQ / 32) {
+        const int g = lane % QF::G, gi = lane / QF::G;
+        T x[QF::CPT][QF::RPT];
 #pragma unroll
-        for (int t = 0; t < RPL; ++t) {
-          const int i = lane + 32 * t;
-          xr[t] = (i < m && i >= j) ? col[i] : T(0);
-          ss += xr[t] * xr[t];
+        for (int q = 0; q < QF::CPT; ++q) {
+          const int col = warp * QF::CW + q * QF::GPW + gi;
+#pragma unroll
+          for (int u = 0; u < QF::RPT; ++u) x[q][u] = T(0);
+          if (col < D) qr_load_v<QF, 0, T>(Xs + (size_t)col * (2 * D), g, x[q]);
         }
-        ss = warp_sum(ss);
-        const T x0 = col[j];
-        __syncwarp();                 // every lane has read the pivot before any lane writes
-        T* vj = vbuf[j % 3];
-        if (ss <= tiny) {
+        // columns (b, be) beyond the right bond of the previous row's tile are zero
+        const int kr = kold[c + 1];
+        auto zero_col = [&](int j) { return (j & (CHI - 1)) >= kr; };
+        const QrOut<T> out{vfwd, false, nullptr, csave, diag};
+        qr_factor<T, 2 * D, D>(x, D, out, lane, warp, zero_col);
+        T mx = 0;
+        for (int j = lane; j < D; j += 32)
+          if (!zero_col(j)) { const T v = diag[j] < 0 ? -diag[j] : diag[j]; mx = v > mx ? v : mx; }
+        mx = warp_max(mx);
+        const T inv = mx > T(0) ? T(1) / mx : T(1);
+        T* Rout = Rstore + (size_t)(c + 1) * D * D;
 #pragma unroll
-          for (int t = 0; t < RPL; ++t) {
-            const int i = lane + 32 * t;
-            if (i < m) { vj[i] = T(0); if (i > j) col[i] = T(0); }
-          }
-          if (lane == 0) vcoef[j % 3] = T(0);
-        } else {
-          const T nrm = num<T>::sqrt_(ss);
-          const T alpha = x0 >= T(0) ? -nrm : nrm;
-          const T v0 = x0 - alpha;
+        for (int q = 0; q < QF::CPT; ++q) {
+          const int col = warp * QF::CW + q * QF::GPW + gi;
+          if (col < D) {
 #pragma unroll
-          for (int t = 0; t < RPL; ++t) {
-            const int i = lane + 32 * t;
-            if (i < m) {
-              vj[i] = (i == j) ? v0 : xr[t];
-              if (i >= j) col[i] = (i == j) ? alpha : T(0);
+            for (int u = 0; u < QF::RPT / 2; ++u) {          // rows below D are zero
+              const int i = g + QF::G * u;
+              const T v = i <= col ? x[q][u] * inv : T(0);
+              if constexpr (!kBig) Rc[col * D + i] = v;      // kBig reads R_{c+1} back from Rstore
+              Rout[col * D + i] = v;
             }
           }
-          if (lane == 0) vcoef[j % 3] = T(1) / (nrm * (nrm + (x0 >= T(0) ? x0 : -x0)));  // 2/|v|^2
         }
-      };
-      // reflector jj applied to one column k (the pivot owner's next column)
-      auto apply1 = [&](int jj, int k) {
-        const T coef = vcoef[jj % 3];
-        if (coef == T(0)) return;
-        const T* v = vbuf[jj % 3];
-        T* col = Xs + (size_t)k * m;
-        T xr[RPL], vr[RPL];
-        T d = 0;
-#pragma unroll
-        for (int t = 0; t < RPL; ++t) {
-          const int i = lane + 32 * t;
-          xr[t] = i < m ? col[i] : T(0);
-          vr[t] = i < m ? v[i] : T(0);
-          d += vr[t] * xr[t];
-        }
-        d = warp_sum(d) * coef;
-#pragma unroll
-        for (int t = 0; t < RPL; ++t) {
-          const int i = lane + 32 * t;
-          if (i < m) col[i] = xr[t] - d * vr[t];
-        }
-      };
-      // reflector jj applied to every column k > lo this warp owns: the dot products of all of
-      // them are reduced in one interleaved butterfly instead of one reduction after another
-      auto apply_batch = [&](int jj, int lo) {
-        const T coef = vcoef[jj % 3];
-        if (coef == T(0)) return;
-        const T* v = vbuf[jj % 3];
-        T vr[RPL], d[CPW];
-#pragma unroll
-        for (int t = 0; t < RPL; ++t) { const int i = lane + 32 * t; vr[t] = i < m ? v[i] : T(0); }
-#pragma unroll
-        for (int q = 0; q < CPW; ++q) {
-          const int k = warp + NWARP * q;
-          d[q] = 0;
-          if (k > lo && k < D) {
-            const T* col = Xs + (size_t)k * m;
-#pragma unroll
-            for (int t = 0; t < RPL; ++t) { const int i = lane + 32 * t; if (i < m) d[q] += vr[t] * col[i]; }
-          }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-          for (int q = 0; q < CPW; ++q) d[q] += __shfl_xor_sync(0xffffffffu, d[q], o);
-#pragma unroll
-        for (int q = 0; q < CPW; ++q) {
-          const int k = warp + NWARP * q;
-          if (k > lo && k < D) {
-            T* col = Xs + (size_t)k * m;
-            const T dc = d[q] * coef;
-#pragma unroll
-            for (int t = 0; t < RPL; ++t) { const int i = lane + 32 * t; if (i < m) col[i] -= dc * vr[t]; }
-          }
-        }
-      };
-      // Step j: the owner of column j+1 applies reflector j to that column and forms reflector
-      // j+1 at once (the critical path), deferring its other columns to the next step; every
-      // other warp applies reflector j to its columns.  Reflectors rotate through three slots,
-      // so a deferred one is still intact when its owner applies it.
-      if (warp == 0) house(0);
-      int pend = -1;                  // reflector this warp still owes its columns > pend + 1
-      for (int j = 0; j < D; ++j) {
-        __syncthreads();
-        if (pend >= 0) { apply_batch(pend, pend + 1); pend = -1; }
-        const int nxt = j + 1;
-        if (nxt < D && warp == nxt % NWARP) {
-          apply1(j, nxt);
-          __syncwarp();
-          house(nxt);
-          pend = j;
-        } else {
-          apply_batch(j, j);
-        }
-        __syncwarp();
-      }
-      __syncthreads();
-      // scale: max |R_jj|; R_{c+1} = X[0:D, :] / scale (col-major), also to Rstore[c+1]
-      if (warp == 0) {
-        T mx = 0;
-        for (int j = lane; j < D; j += 32) { T v = Xs[(size_t)j * m + j]; v = v < 0 ? -v : v; mx = v > mx ? v : mx; }
-        mx = warp_max(mx);
-        if (lane == 0) red[0] = mx > T(0) ? T(1) / mx : T(1);
-      }
-      __syncthreads();
-      const T inv = red[0];
-      T* Rout = Rstore + (size_t)(c + 1) * D * D;
-      for (int e = tid; e < D * D; e += NT) {
-        const int i = e % D, j = e / D;
-        const T v = (i <= j) ? Xs[(size_t)j * m + i] * inv : T(0);
-        if constexpr (!kBig) Rc[e] = v;      // kBig reads R_{c+1} back from Rstore
-        Rout[e] = v;
       }
       __syncthreads();
     }
@@ -714,16 +696,13 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
 #pragma unroll
           for (int jj = 0; jj < 4; ++jj) {
             if (j0 + jj < n) {
-              const T col4[4] = {acc[0][jj], acc[1][jj], acc[2][jj], acc[3][jj]};
-              st4(Yc + (size_t)(j0 + jj) * DP + i0, col4);
 #pragma unroll
-              for (int ii = 0; ii < 4; ++ii) fro += acc[ii][jj] * acc[ii][jj];
+              for (int ii = 0; ii < 4; ++ii) {
+                Yc[(size_t)(j0 + jj) * DP + qr_pos<QB::G>(i0 + ii)] = acc[ii][jj];
+                fro += acc[ii][jj] * acc[ii][jj];
+              }
             }
           }
-        }
-        if constexpr (DP > D) {
-          constexpr int PAD = DP > D ? DP - D : 1;
-          for (int e = tid; e < PAD * n; e += NT) Yc[(size_t)(e / PAD) * DP + D + e % PAD] = T(0);
         }
       }
       // the Jacobi runs on npad = n rounded up to 8 columns (blocks of 4, an even number of
@@ -755,17 +734,56 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
         // smaller 99.9th percentile of the conditional error).  Q1 is not kept; Q2's reflectors
         // overwrite R_c (shared memory, or its slot of the global R store for CHI = 64: R_c is
         // not read again in this row), their coefficients go to csave.
-        householder_r<T, D, D, NWARP>(Yc, DP, n, reinterpret_cast<T (*)[D]>(Vc), vcoef, nullptr, nullptr, lane, warp);
-        for (int e = tid; e < DP * n; e += NT) {           // R1^T, rows n..DP-1 zero
-          const int i = e % DP, j = e / DP;
-          Vc[e] = (i < n && j <= i) ? Yc[(size_t)i * DP + j] : T(0);
-        }
-        householder_r<T, D, D, NWARP>(Vc, DP, n, reinterpret_cast<T (*)[D]>(Yc), vcoef, Rc, csave, lane, warp);
-        for (int e = tid; e < DP * npad; e += NT) {        // R2^T in Y, zero outside n x n
-          const int i = e % DP, j = e / DP;
-          Yc[e] = (i < n && j < n && j <= i) ? Vc[(size_t)i * DP + j] : T(0);
+        auto none = [](int) { return false; };
+        const int g = lane % QB::G, gi = lane / QB::G;
+        T x[QB::CPT][QB::RPT];
+        auto load = [&](const T* A) {
+#pragma unroll
+          for (int q = 0; q < QB::CPT; ++q) {
+            const int col = warp * QB::CW + q * QB::GPW + gi;
+#pragma unroll
+            for (int u = 0; u < QB::RPT; ++u) x[q][u] = T(0);
+            if (col < n) qr_load_v<QB, 0, T>(A + (size_t)col * DP, g, x[q]);
+          }
+        };
+        if (warp < QB::NTQ / 32) {
+          load(Yc);
+          if constexpr (QB::NTQ == 32) __syncwarp();
+          else named_barrier(10, QB::NTQ);
+          const QrOut<T> out1{kBig ? vfwd : Yc, false, nullptr, csave, diag};
+          qr_factor<T, D, D>(x, n, out1, lane, warp, none);
+#pragma unroll
+          for (int q = 0; q < QB::CPT; ++q) {                // R1^T, stored for the next factorisation
+            const int col = warp * QB::CW + q * QB::GPW + gi;
+            if (col < D) {
+#pragma unroll
+              for (int u = 0; u < QB::RPT; ++u) {
+                const int i = g + QB::G * u;
+                Vc[(size_t)i * DP + qr_pos<QB::G>(col)] = (i <= col && col < n) ? x[q][u] : T(0);
+              }
+            }
+          }
+          if constexpr (QB::NTQ == 32) __syncwarp();
+          else named_barrier(10, QB::NTQ);
+          load(Vc);
+          const QrOut<T> out2{kBig ? vfwd : Rc, !kBig, kBig ? Rc : nullptr, csave, diag};
+          qr_factor<T, D, D>(x, n, out2, lane, warp, none);
+#pragma unroll
+          for (int q = 0; q < QB::CPT; ++q) {                // R2^T in Y, zero outside n x n
+            const int col = warp * QB::CW + q * QB::GPW + gi;
+            if (col < D) {
+#pragma unroll
+              for (int u = 0; u < QB::RPT; ++u) {
+                const int i = g + QB::G * u;
+                Yc[(size_t)i * DP + col] = (i <= col && col < n) ? x[q][u] : T(0);
+              }
+            }
+          }
+          if constexpr (DP > D)
+            for (int e = tid; e < (DP - D) * D; e += QB::NTQ) Yc[(size_t)(e / (DP - D)) * DP + D + e % (DP - D)] = T(0);
         }
         __syncthreads();
+        if (sizeof(T) == 4 && tid < n) { const T den = csave[tid]; csave[tid] = den == T(0) ? den : T(1) / den; }
         for (int e = tid; e < DP * npad; e += NT) { const int i = e % DP, j = e / DP; Vc[e] = (i == j) ? T(1) : T(0); }
         __syncthreads();
       }
@@ -928,49 +946,21 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
         // V_k = Q2 Z_sel = H_0 H_1 ... H_{n-1} Z_sel: each warp takes its selected columns into
         // registers, applies the reflectors from the last to the first, and writes the result to
         // column g of V (the selection becomes the identity)
-        constexpr int RPL = D / 32 > 0 ? D / 32 : 1;
-        constexpr int CPQ = (CHI + NWARP - 1) / NWARP;
-        T xz[CPQ][RPL];
+        const int g = lane % QB::G, col = warp * QB::GPW + lane / QB::G;
+        const bool mine = col < k;
+        T xz[QB::RPT];
 #pragma unroll
-        for (int q = 0; q < CPQ; ++q) {
-          const int g = warp + NWARP * q;
-#pragma unroll
-          for (int t = 0; t < RPL; ++t) {
-            const int i = lane + 32 * t;
-            xz[q][t] = (g < k && i < n) ? Vc[(size_t)sel[g] * DP + i] : T(0);
-          }
+        for (int u = 0; u < QB::RPT; ++u) {
+          const int i = g + QB::G * u;
+          xz[u] = (mine && i < n) ? Vc[(size_t)sel[col] * DP + i] : T(0);
         }
         __syncthreads();
-        for (int j = n - 1; j >= 0; --j) {
-          const T coef = csave[j];
-          if (coef == T(0)) continue;
-          T vr[RPL], d[CPQ];
+        if (warp * QB::GPW < k) {
+          qr_apply_q<T, D, D>(xz, n, Rc, csave, g);
 #pragma unroll
-          for (int t = 0; t < RPL; ++t) { const int i = lane + 32 * t; vr[t] = (i < n) ? Rc[(size_t)j * D + i] : T(0); }
-#pragma unroll
-          for (int q = 0; q < CPQ; ++q) {
-            d[q] = 0;
-#pragma unroll
-            for (int t = 0; t < RPL; ++t) d[q] += vr[t] * xz[q][t];
-          }
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-            for (int q = 0; q < CPQ; ++q) d[q] += __shfl_xor_sync(0xffffffffu, d[q], o);
-#pragma unroll
-          for (int q = 0; q < CPQ; ++q) {
-            const T dc = d[q] * coef;
-#pragma unroll
-            for (int t = 0; t < RPL; ++t) xz[q][t] -= dc * vr[t];
-          }
-        }
-#pragma unroll
-        for (int q = 0; q < CPQ; ++q) {
-          const int g = warp + NWARP * q;
-#pragma unroll
-          for (int t = 0; t < RPL; ++t) {
-            const int i = lane + 32 * t;
-            if (g < k && i < n) Vc[(size_t)g * DP + i] = xz[q][t];
+          for (int u = 0; u < QB::RPT; ++u) {
+            const int i = g + QB::G * u;
+            if (mine && i < n) Vc[(size_t)col * DP + i] = xz[u];
           }
         }
         __syncthreads();
