@@ -44,17 +44,40 @@ template <typename T, int D> __device__ __forceinline__ T jacobi_tol() {
 template <typename T> struct Vec16;
 template <> struct Vec16<float> { using type = float4; };
 template <> struct Vec16<double> { using type = double2; };
-__device__ __forceinline__ float dot16(const float4& a, const float4& b) { return a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w; }
-__device__ __forceinline__ double dot16(const double2& a, const double2& b) { return a.x * b.x + a.y * b.y; }
+// Which product of a sum is rounded before it enters a fused multiply-add is written out, so that
+// the results do not hang on how the compiler contracts each place.
+__device__ __forceinline__ float dot16(const float4& a, const float4& b) {
+  return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.x, b.x, __fmul_rn(a.y, b.y))));
+}
+__device__ __forceinline__ double dot16(const double2& a, const double2& b) {
+  return fma(a.x, b.x, __dmul_rn(a.y, b.y));
+}
+// the square of a vector with the other product rounded first
+__device__ __forceinline__ float sq16(const float4& a) {
+  return fmaf(a.w, a.w, fmaf(a.z, a.z, fmaf(a.y, a.y, __fmul_rn(a.x, a.x))));
+}
+__device__ __forceinline__ double sq16(const double2& a) { return fma(a.y, a.y, __dmul_rn(a.x, a.x)); }
+__device__ __forceinline__ float rot_u(float a, float b, float c, float s) {
+  return fmaf(c, a, -__fmul_rn(s, b));
+}
+__device__ __forceinline__ float rot_v(float a, float b, float c, float s) {
+  return fmaf(s, a, __fmul_rn(c, b));
+}
+__device__ __forceinline__ double rot_u(double a, double b, double c, double s) {
+  return fma(c, a, -__dmul_rn(s, b));
+}
+__device__ __forceinline__ double rot_v(double a, double b, double c, double s) {
+  return fma(s, a, __dmul_rn(c, b));
+}
 __device__ __forceinline__ void rot16(float4& u, float4& v, float c, float s) {
   const float4 a = u, b = v;
-  u = make_float4(c * a.x - s * b.x, c * a.y - s * b.y, c * a.z - s * b.z, c * a.w - s * b.w);
-  v = make_float4(s * a.x + c * b.x, s * a.y + c * b.y, s * a.z + c * b.z, s * a.w + c * b.w);
+  u = make_float4(rot_u(a.x, b.x, c, s), rot_u(a.y, b.y, c, s), rot_u(a.z, b.z, c, s), rot_u(a.w, b.w, c, s));
+  v = make_float4(rot_v(a.x, b.x, c, s), rot_v(a.y, b.y, c, s), rot_v(a.z, b.z, c, s), rot_v(a.w, b.w, c, s));
 }
 __device__ __forceinline__ void rot16(double2& u, double2& v, double c, double s) {
   const double2 a = u, b = v;
-  u = make_double2(c * a.x - s * b.x, c * a.y - s * b.y);
-  v = make_double2(s * a.x + c * b.x, s * a.y + c * b.y);
+  u = make_double2(rot_u(a.x, b.x, c, s), rot_u(a.y, b.y, c, s));
+  v = make_double2(rot_v(a.x, b.x, c, s), rot_v(a.y, b.y, c, s));
 }
 // Jacobi rotation (c, s) that makes columns p, q orthogonal, from a = |y_p|^2, b = |y_q|^2,
 // g = y_p . y_q (y_p' = c y_p - s y_q, y_q' = s y_p + c y_q).  The angle solves
@@ -796,8 +819,15 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
       // pair of columns meets once per sweep; the columns a warp touches in a block-round are
       // its own, so sub-rounds are ordered by __syncwarp and only block-rounds need the
       // CTA-wide barrier (NB-1 per sweep instead of npad-1).  8 lanes per pair, each lane
-      // holding DP/8 rows of both columns in 16-byte vectors; the three dot products of a pair
-      // are reduced together over the 8 lanes.
+      // holding DP/8 rows of both columns in 16-byte vectors.
+      // Few pairs rotate: columns below tinyY never do (nor grow, so a block without a column
+      // above it is left out for good), and of the others on the preconditioned matrix in FP32
+      // about 70, 40, 6 and 0 of 2016 in the sweeps of a chi = 32 site, in 7.5, 6.2, 1.6 and 0.2 of
+      // 91 block pairs (measured).  So a warp first tests its 16 pairs side by side, which is the
+      // whole work of a block pair without rotations, and enters the sub-rounds at the first pair
+      // that rotates; block-rounds without a live block pair are skipped, barrier and all.
+      // 65 -> 27 thousand cycles a site at chi = 32 (L = 32); the build 150 -> 130 us a site step
+      // with one realization per SM, 214 -> 172 with three.
       constexpr int NJ = 8 * CHI;
       constexpr int VEC = JStride<T, CHI>::VEC;
       constexpr int NV = DP / (8 * VEC);
@@ -806,47 +836,71 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
       if (tid < NJ) {
         const int wj = tid >> 5, grp = (tid >> 3) & 3, li = tid & 7;
         const int NB = npad / 4, mb = NB - 1;
-        const bool wact = wj < NB / 2;
-        // The sweep is bound by shared-memory traffic at the occupancy the build runs at, so a
-        // pair's V columns are read only when the pair rotates, and in the cross sub-rounds
-        // each 8-lane group keeps its block-A column (Y and V) in registers.
-        auto rotation = [&](const V16* u, const V16* w, T& cs, T& sn) -> bool {
-          T g = 0, a = 0, b = 0;
+        auto dot = [&](const V16* u, const V16* w) {
+          T g = 0;
 #pragma unroll
-          for (int k = 0; k < NV; ++k) {
-            g += dot16(u[k], w[k]);
-            a += dot16(u[k], u[k]);
-            b += dot16(w[k], w[k]);
-          }
-          g = group8_sum(g); a = group8_sum(a); b = group8_sum(b);
-          if (a > tinyY && b > tinyY && g * g > tol * tol * a * b) {
-            rotation_from_gram(a, b, g, cs, sn);
-            return true;
-          }
-          return false;
+          for (int k = 0; k < NV; ++k) g += dot16(u[k], w[k]);
+          return g;
         };
-        auto jpair = [&](int p, int q) {          // both columns from shared memory
-          V16* yp = reinterpret_cast<V16*>(Yc + (size_t)p * DP);
-          V16* yq = reinterpret_cast<V16*>(Yc + (size_t)q * DP);
+        // squared norm of a block-A column: with one vector per lane the other product of the
+        // first two is the one rounded
+        auto norm_a = [&](const V16* u) { return NV == 1 ? sq16(u[0]) : dot(u, u); };
+        auto col = [&](T* base, int p) { return reinterpret_cast<V16*>(base + (size_t)p * DP) + li; };
+        auto get = [&](V16* c, V16* u) {
+#pragma unroll
+          for (int k = 0; k < NV; ++k) u[k] = c[8 * k];
+        };
+        auto put = [&](V16* c, const V16* u) {
+#pragma unroll
+          for (int k = 0; k < NV; ++k) c[8 * k] = u[k];
+        };
+        // sums over the 8 lanes of a group, all values in step
+        auto sum8 = [&](T* v, int n) {
+#pragma unroll
+          for (int o = 1; o <= 4; o <<= 1)
+#pragma unroll
+            for (int t = 0; t < n; ++t) v[t] += __shfl_xor_sync(0xffffffffu, v[t], o);
+        };
+        auto rotates = [&](T a, T b, T g) { return a > tinyY && b > tinyY && g * g > tol * tol * a * b; };
+        // blocks with a column above tinyY (n2: the columns' squared norms; warp-uniform loops: the
+        // shuffles need the whole warp)
+        T* const n2 = sig;
+        for (int p0 = wj * 4; p0 < npad; p0 += NJ / 8) {
+          V16 u[NV];
+          get(col(Yc, p0 + grp), u);
+          T a[2] = {dot(u, u), norm_a(u)};
+          sum8(a, 2);
+          if (li == 0) n2[p0 + grp] = a[0] > a[1] ? a[0] : a[1];
+        }
+        named_barrier(1, NJ);
+        bool live = false;
+        if (lane < NB) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) live |= n2[4 * lane + i] > tinyY;
+        }
+        const unsigned blocks = __ballot_sync(0xffffffffu, live);
+        // block pair of slot w in block-round br (circle method: slot 0 keeps block NB-1)
+        auto slot_pair = [&](int br, int w, int& bA, int& bB) {
+          bA = w == 0 ? NB - 1 : (br + w >= mb ? br + w - mb : br + w);
+          bB = w == 0 ? br : (br >= w ? br - w : br - w + mb);
+        };
+        // one pair from shared memory (inside a block)
+        auto jpair = [&](int p, int q) {
           V16 up[NV], uq[NV];
-#pragma unroll
-          for (int k = 0; k < NV; ++k) { up[k] = yp[li + 8 * k]; uq[k] = yq[li + 8 * k]; }
-          T cs, sn;
-          if (rotation(up, uq, cs, sn)) {
-            V16* vp = reinterpret_cast<V16*>(Vc + (size_t)p * DP);
-            V16* vq = reinterpret_cast<V16*>(Vc + (size_t)q * DP);
+          get(col(Yc, p), up);
+          get(col(Yc, q), uq);
+          T v[3] = {dot(up, uq), dot(up, up), dot(uq, uq)};
+          sum8(v, 3);
+          if (rotates(v[1], v[2], v[0])) {
+            T cs, sn;
+            rotation_from_gram(v[1], v[2], v[0], cs, sn);
             V16 wp[NV], wq[NV];
+            get(col(Vc, p), wp);
+            get(col(Vc, q), wq);
 #pragma unroll
-            for (int k = 0; k < NV; ++k) { wp[k] = vp[li + 8 * k]; wq[k] = vq[li + 8 * k]; }
-#pragma unroll
-            for (int k = 0; k < NV; ++k) {
-              rot16(up[k], uq[k], cs, sn);
-              rot16(wp[k], wq[k], cs, sn);
-              yp[li + 8 * k] = up[k];
-              yq[li + 8 * k] = uq[k];
-              vp[li + 8 * k] = wp[k];
-              vq[li + 8 * k] = wq[k];
-            }
+            for (int k = 0; k < NV; ++k) { rot16(up[k], uq[k], cs, sn); rot16(wp[k], wq[k], cs, sn); }
+            put(col(Yc, p), up); put(col(Yc, q), uq);
+            put(col(Vc, p), wp); put(col(Vc, q), wq);
             if (li == 0) rot[sweep % 3] = 1;
           }
         };
@@ -856,11 +910,13 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
           // thread read a flag that was already cleared and leave the loop alone)
           if (tid == 0) rot[(sweep + 1) % 3] = 0;
           for (int br = 0; br < mb; ++br) {
-            if (wact) {       // warp-uniform: the shuffles of the reductions need the whole warp
-              // block pair of slot wj (circle method: slot 0 keeps block NB-1)
-              const int bA = wj == 0 ? NB - 1 : (br + wj) % mb;
-              const int bB = wj == 0 ? br : (br - wj + mb) % mb;
-              if (br == 0) {
+            int bA = 0, bB = 0;
+            slot_pair(br, lane < NB / 2 ? lane : 0, bA, bB);
+            const unsigned busy = __ballot_sync(0xffffffffu, lane < NB / 2 && ((blocks >> bA) & (blocks >> bB) & 1u));
+            if (br > 0 && busy == 0) continue;         // no live block pair: the same in every warp
+            if (wj < NB / 2) {
+              slot_pair(br, wj, bA, bB);
+              if (br == 0 && (((blocks >> bA) | (blocks >> bB)) & 1u)) {
                 // pairs inside blocks A (groups 0, 1) and B (groups 2, 3):
                 // {(0,1),(2,3)}, {(0,2),(1,3)}, {(0,3),(1,2)}
                 const int blk = 4 * ((grp < 2) ? bA : bB), gi = grp & 1;
@@ -872,47 +928,61 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
                   __syncwarp();
                 }
               }
-              // cross pairs: group grp holds column A = 4 bA + grp and meets the four columns
-              // of block B in turn (B column (grp + t) mod 4 in sub-round t)
-              const int pa = 4 * bA + grp;
-              V16* ya_s = reinterpret_cast<V16*>(Yc + (size_t)pa * DP);
-              V16* va_s = reinterpret_cast<V16*>(Vc + (size_t)pa * DP);
-              V16 ya[NV], va[NV];
+              if ((busy >> wj) & 1u) {
+                // cross pairs: group grp holds column A = 4 bA + grp and meets the four columns
+                // of block B in turn (B column (grp + t) mod 4 in sub-round t)
+                const int pa = 4 * bA + grp;
+                V16 ya[NV], va[NV];
+                get(col(Yc, pa), ya);
+                int t0 = 0;
+                // The test pays where few block pairs rotate: on the preconditioned matrix in FP32
+                // at once, on the zip-up's M (a third of the block pairs in the first sweep, an
+                // eighth in the fifth) from the sixth sweep on (L = 48, chi = 32: 277 ms, from the
+                // third 288, never 288), in FP64, whose tolerance asks for more rotations, from the
+                // third on.
+                if (sizeof(T) == 8 ? sweep >= 2 : (!zip || sweep >= 5)) {
+                  T v[9];               // A's norm, four products, the four norms of block B
+                  v[0] = norm_a(ya);
 #pragma unroll
-              for (int k = 0; k < NV; ++k) ya[k] = ya_s[li + 8 * k];
-              bool va_held = false;   // group-uniform: every lane of a group sees the same sums
-#pragma unroll 1
-              for (int t = 0; t < 4; ++t) {
-                const int q = 4 * bB + ((grp + t) & 3);
-                V16* yq = reinterpret_cast<V16*>(Yc + (size_t)q * DP);
-                V16 uq[NV];
-#pragma unroll
-                for (int k = 0; k < NV; ++k) uq[k] = yq[li + 8 * k];
-                T cs, sn;
-                if (rotation(ya, uq, cs, sn)) {
-                  V16* vq = reinterpret_cast<V16*>(Vc + (size_t)q * DP);
-                  V16 wq[NV];
-                  if (!va_held) {
-#pragma unroll
-                    for (int k = 0; k < NV; ++k) va[k] = va_s[li + 8 * k];
-                    va_held = true;
+                  for (int t = 0; t < 4; ++t) {
+                    V16 uq[NV];
+                    get(col(Yc, 4 * bB + ((grp + t) & 3)), uq);
+                    v[1 + t] = dot(ya, uq);
+                    v[5 + t] = dot(uq, uq);
                   }
+                  sum8(v, 9);
+                  unsigned hit = 0;
 #pragma unroll
-                  for (int k = 0; k < NV; ++k) wq[k] = vq[li + 8 * k];
-#pragma unroll
-                  for (int k = 0; k < NV; ++k) {
-                    rot16(ya[k], uq[k], cs, sn);
-                    rot16(va[k], wq[k], cs, sn);
-                    yq[li + 8 * k] = uq[k];
-                    vq[li + 8 * k] = wq[k];
-                  }
-                  if (li == 0) rot[sweep % 3] = 1;
+                  for (int t = 0; t < 4; ++t) hit |= rotates(v[0], v[5 + t], v[1 + t]) ? 1u << t : 0u;
+                  hit = __reduce_or_sync(0xffffffffu, hit);
+                  t0 = hit ? __ffs(hit) - 1 : 4;
                 }
-                __syncwarp();
-              }
-              if (va_held) {          // column A changed: back to shared memory
+                bool va_held = false;   // group-uniform: every lane of a group sees the same sums
+#pragma unroll 1
+                for (int t = t0; t < 4; ++t) {
+                  const int q = 4 * bB + ((grp + t) & 3);
+                  V16 uq[NV];
+                  get(col(Yc, q), uq);
+                  T v[3] = {dot(ya, uq), norm_a(ya), dot(uq, uq)};
+                  sum8(v, 3);
+                  if (rotates(v[1], v[2], v[0])) {
+                    T cs, sn;
+                    rotation_from_gram(v[1], v[2], v[0], cs, sn);
+                    V16 wq[NV];
+                    if (!va_held) { get(col(Vc, pa), va); va_held = true; }
+                    get(col(Vc, q), wq);
 #pragma unroll
-                for (int k = 0; k < NV; ++k) { ya_s[li + 8 * k] = ya[k]; va_s[li + 8 * k] = va[k]; }
+                    for (int k = 0; k < NV; ++k) { rot16(ya[k], uq[k], cs, sn); rot16(va[k], wq[k], cs, sn); }
+                    put(col(Yc, q), uq);
+                    put(col(Vc, q), wq);
+                    if (li == 0) rot[sweep % 3] = 1;
+                  }
+                  __syncwarp();
+                }
+                if (va_held) {          // column A changed: back to shared memory
+                  put(col(Yc, pa), ya);
+                  put(col(Vc, pa), va);
+                }
               }
             }
             named_barrier(1, NJ);
