@@ -16,8 +16,23 @@
 // 1e-3 conditional tolerance because the contraction of a sign-indefinite MPS amplifies
 // operand rounding.
 //
-// Shared-memory operands use the K-major, no-swizzle canonical layout: 8-row x 16-byte
-// core matrices, 128 B apart along K (LBO) and 32*CHI B apart along M/N (SBO).
+// Roles (256 threads): warps 0-3 own the proposals, warp 4 issues the MMAs, warps 5-7 load the
+// environment tiles ahead of time, split them and lay them out.  The A operand lives in tensor
+// memory: a proposal's thread writes its row there with tcgen05.st, next to the accumulator it
+// reads back, so it never passes through shared memory.  B operands use the K-major, no-swizzle
+// canonical layout: 8-row x 16-byte core matrices, 128 B apart along K (LBO) and 32*CHI B apart
+// along N (SBO); the two y of a site are adjacent, so the left sweep, whose A is the same for both,
+// takes them in one MMA of N = 2 CHI.
+//
+// What bounds it: at CHI = 32 the right vectors R_{c+1}, 32 KB per site and tile written in the right
+// sweep and read back in the left one (5.1 TB/s of them at L = 64 with two tiles on every SM, of 6.8
+// measured for a copy); at CHI = 16 the instructions of the proposal warps.  They are kept
+// [site][y][j/4][proposal][4], so every access is 512 contiguous bytes a warp (one row per proposal
+// kept the load/store unit busy 32 lines an instruction), and the left sweep copies the next site's
+// into shared memory while it finishes this one.  The loops over the columns are not unrolled: with
+// straight-line bodies the warps waited for instructions three cycles an issue.
+// One GB300, propose() before and now: CHI = 32, L = 64, 64 realizations x 1000 proposals 92 -> 38 ms;
+// L = 48, 448 x 500 158 -> 65 ms; CHI = 16, L = 32, 1024 x 2000 246 -> 140 ms.
 #include "common.cuh"
 #include "kernels.h"
 
@@ -43,54 +58,80 @@ __host__ __device__ constexpr uint32_t idesc_tf32() {
   return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-__device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t ad, uint64_t bd, uint32_t idesc, uint32_t acc) {
-  asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}\n"
-               ::"r"(d_tmem), "l"(ad), "l"(bd), "r"(idesc), "r"(acc));
+// D (tensor memory) = A (tensor memory, K columns from a_tmem) B (shared memory) [+ D]
+__device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint32_t a_tmem, uint64_t bd, uint32_t idesc, uint32_t acc) {
+  asm volatile("{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\ntcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n}\n"
+               ::"r"(d_tmem), "r"(a_tmem), "l"(bd), "r"(idesc), "r"(acc));
 }
 __device__ __forceinline__ void mma_commit(uint64_t* mbar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(su32(mbar)));
 }
+__device__ __forceinline__ bool try_parity(uint64_t* mbar, uint32_t parity) {
+  uint32_t done = 0;
+  asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
+               : "=r"(done) : "r"(su32(mbar)), "r"(parity) : "memory");
+  return done != 0;
+}
 // Bounded wait for the given phase parity; false when the limit ran out.
 __device__ __forceinline__ bool wait_parity(uint64_t* mbar, uint32_t parity, long long limit = 1ll << 20) {
-  uint32_t done = 0;
-  for (long long it = 0; it < limit && !done; ++it) {
-    asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}\n"
-                 : "=r"(done) : "r"(su32(mbar)), "r"(parity) : "memory");
-  }
-  return done != 0;
+  for (long long it = 0; it < limit; ++it)
+    if (try_parity(mbar, parity)) return true;
+  return false;
+}
+// One lane of a converged warp.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0;
+}
+// Barrier id over NTHR threads that tells each whether any of them passed true.
+template <int NTHR> __device__ __forceinline__ bool any_of(int id, bool v) {
+  uint32_t r;
+  asm volatile("{\n.reg .pred p, q;\nsetp.ne.u32 p, %1, 0;\nbarrier.cta.red.or.pred q, %2, %3, p;\nselp.u32 %0, 1, 0, q;\n}\n"
+               : "=r"(r) : "r"((uint32_t)v), "r"(id), "n"(NTHR) : "memory");
+  return r != 0;
+}
+__device__ __forceinline__ void mbar_init(uint64_t* mbar, uint32_t count) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(mbar)), "r"(count));
+}
+__device__ __forceinline__ void mbar_arrive(uint64_t* mbar) {
+  asm volatile("{\n.reg .b64 st;\nmbarrier.arrive.shared::cta.b64 st, [%0];\n}\n" ::"r"(su32(mbar)) : "memory");
 }
 __device__ __forceinline__ void fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-template <int NC> struct TmemLd;
-template <> struct TmemLd<32> {
-  static __device__ __forceinline__ void ld(uint32_t ta, float* v) {
-    uint32_t r[32];
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-                 "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-                   "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-                   "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-                 : "r"(ta));
+// 8 columns of this thread's TMEM lane
+__device__ __forceinline__ void tmem_ld8(uint32_t ta, float* v) {
+  uint32_t r[8];
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(ta));
 #pragma unroll
-    for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
-  }
-};
-template <> struct TmemLd<16> {
-  static __device__ __forceinline__ void ld(uint32_t ta, float* v) {
-    uint32_t r[16];
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-                 : "r"(ta));
+  for (int j = 0; j < 8; ++j) v[j] = __uint_as_float(r[j]);
+}
+__device__ __forceinline__ void tmem_st8(uint32_t ta, const float* v) {
+  uint32_t r[8];
 #pragma unroll
-    for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
-  }
-};
+  for (int j = 0; j < 8; ++j) r[j] = __float_as_uint(v[j]);
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%8], {%0,%1,%2,%3,%4,%5,%6,%7};"
+               ::"r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(ta)
+               : "memory");
+}
+__device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
+// The same rounding of a finite x below the largest binade, in two integer operations: half of
+// the 11-bit significand's last place is added to the magnitude and the rest cut off (checked against
+// the instruction for every such float).  cvt.rna takes four issue slots.
+__device__ __forceinline__ float tf32_rna_finite(float x) {
+  return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xffffe000u);
+}
+__device__ __forceinline__ float max_nan(float a, float b) {       // NaN if either is
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
 __device__ __forceinline__ float tf32_rna(float x) {
   uint32_t r;
   asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
@@ -102,55 +143,87 @@ template <int KD> __device__ __forceinline__ int koff(int r, int k) {
   return (r >> 3) * (8 * KD) + (k >> 2) * 32 + (r & 7) * 4 + (k & 3);
 }
 
-// Write this thread's row (CHI values) of an A operand as hi/lo TF32 parts.
-template <int CHI>
-__device__ __forceinline__ void put_row_split(float* hi, float* lo, int m, const float* x) {
+// Write eight values of this thread's row of an A operand: hi parts at ta, lo parts CHI columns on.
+// fin (warp-uniform): all of them are finite.
+template <int CHI> __device__ __forceinline__ void put8_split(uint32_t ta, const float* x, bool fin) {
+  float h[8], l[8];
+  if (fin) {
 #pragma unroll
-  for (int kg = 0; kg < CHI / 4; ++kg) {
-    float h[4], l[4];
+    for (int t = 0; t < 8; ++t) { h[t] = tf32_rna_finite(x[t]); l[t] = tf32_rna_finite(x[t] - h[t]); }
+  } else {
 #pragma unroll
-    for (int t = 0; t < 4; ++t) { h[t] = tf32_rna(x[4 * kg + t]); l[t] = tf32_rna(x[4 * kg + t] - h[t]); }
-    const int o = koff<CHI>(m, 4 * kg);
-    *reinterpret_cast<float4*>(hi + o) = make_float4(h[0], h[1], h[2], h[3]);
-    *reinterpret_cast<float4*>(lo + o) = make_float4(l[0], l[1], l[2], l[3]);
+    for (int t = 0; t < 8; ++t) { h[t] = tf32_rna(x[t]); l[t] = tf32_rna(x[t] - h[t]); }
+  }
+  tmem_st8(ta, h);
+  tmem_st8(ta + CHI, l);
+}
+// The row (1, 0, ..., 0) that a sweep starts from.
+template <int CHI> __device__ __forceinline__ void put_e0(uint32_t ta) {
+#pragma unroll 1
+  for (int j = 0; j < 2 * CHI; j += 8) {
+    const float x[8] = {j == 0 ? 1.0f : 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    tmem_st8(ta + j, x);
   }
 }
+
+// Draw s = +1 iff u < q(+), u = m53 2^-53: m < ceil(q 2^53) exactly, in integers.
+__device__ __forceinline__ bool draw_below(uint64_t m53, float q) {
+  if (q >= 1.0f) return true;
+  if (!(q > 0.0f)) return false;
+  const uint32_t bits = __float_as_uint(q);
+  const int ex = (int)((bits >> 23) & 0xffu);
+  const uint64_t mant = (ex == 0) ? (uint64_t)(bits & 0x7fffffu) : (uint64_t)((bits & 0x7fffffu) | 0x800000u);
+  const int sh = (ex == 0 ? 1 : ex) - 150 + 53;
+  uint64_t C;
+  if (sh >= 0) C = mant << sh;
+  else { const int k = -sh; C = (k >= 64) ? 1ull : ((mant + ((1ull << k) - 1ull)) >> k); }
+  return m53 < C;
+}
+
+template <int CHI> struct Cfg {
+  static constexpr int NT = 256;                    // 4 proposal warps, 1 MMA warp, 3 tile warps
+  static constexpr int NPROD = 96;
+  static constexpr int BOP = CHI * CHI;             // floats of one B operand
+  static constexpr int TILE = 2 * BOP;              // floats of one cached site tile [y][al][be]
+  static constexpr int STAGE = 4 * BOP;             // [hi y0, hi y1, lo y0, lo y1]
+  static constexpr int NST = CHI <= 16 ? 4 : 3;     // stages
+  static constexpr int RAWTILE = 2 * CHI * (CHI + 4);
+  // tensor memory: accumulators of y = 0, 1, then the A rows R0 (or l) hi, lo, R1 hi, lo
+  static constexpr int TCOLS = 6 * CHI <= 128 ? 128 : 256;
+  // CTAs per SM: tensor memory and registers allow two at CHI = 32, three at 16
+  static constexpr int PER_SM = CHI <= 16 ? 3 : 2;
+};
 
 }  // namespace tc
 
 template <int CHI>
-__global__ void __launch_bounds__(128) sample_tc_kernel(SampleArgs a) {
+__global__ void __launch_bounds__(tc::Cfg<CHI>::NT, tc::Cfg<CHI>::PER_SM) sample_tc_kernel(SampleArgs a, int raw_tiles) {
   using namespace tc;
-  constexpr int AOP = M * CHI;            // floats of one A operand
-  constexpr int BOP = CHI * CHI;          // floats of one B operand
-  constexpr int TILE = 2 * CHI * CHI;     // floats of one cached site tile [y][al][be]
-  constexpr int PRE = TILE / M;           // tile floats each thread prefetches
-  constexpr int KSTEPS = CHI / 8;
+  using C = Cfg<CHI>;
+  constexpr int BOP = C::BOP, TILE = C::TILE, NST = C::NST;
   constexpr uint32_t SBO = 32 * CHI;      // bytes between 8-row groups (K = CHI)
-  constexpr uint32_t IDESC = idesc_tf32<CHI>();
-  constexpr int TCOLS = 2 * CHI < 32 ? 32 : 2 * CHI;
   const int L = a.L, N = L * L;
   const int tid = threadIdx.x, warp = tid >> 5;
-  const int words_row = (L + 31) / 32;
 
   extern __shared__ __align__(1024) float smf[];
-  float* Abuf = smf;                                  // 4 operands: [0]=R0/l hi [1]=R0/l lo [2]=R1 hi [3]=R1 lo
-  float* Bbuf = Abuf + 4 * AOP;                       // [stage][y][hi,lo]
+  float* Bbuf = smf;                                  // [stage][hi y0, hi y1, lo y0, lo y1]
   const int LP = (L + 15) & ~15;                      // keeps the uint32 arrays 16-byte aligned
-  int8_t* jh_s = reinterpret_cast<int8_t*>(Bbuf + 8 * BOP);
-  int8_t* jv_s = jh_s + LP;
-  uint32_t* prow = reinterpret_cast<uint32_t*>(jv_s + LP);              // [words_row][M]
-  uint32_t* crow = prow + (size_t)words_row * M;
-  __shared__ __align__(8) uint64_t mbar;
+  float* Rawbuf = Bbuf + NST * C::STAGE;              // [buffer][y, al][be], rows padded
+  float* Rws = Rawbuf + raw_tiles * C::RAWTILE;          // [y][j / 4][proposal][4]
+  int8_t* jrow = reinterpret_cast<int8_t*>(Rws + 2 * CHI * M);      // [proposal warp][Jh row, Jv row above]
+  uint32_t* prow = reinterpret_cast<uint32_t*>(jrow + 8 * LP);          // [words_row][M]
+  __shared__ __align__(8) uint64_t bar_a, bar_d, bar_full[NST], bar_free[NST];
   __shared__ uint32_t tslot;
-  __shared__ int abort_flag;
+  __shared__ volatile int abort_flag;
 
   if (warp == 0) {
-    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&tslot)), "r"(TCOLS));
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(&tslot)), "r"(C::TCOLS));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
   }
   if (tid == 0) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(&mbar)), "r"(1));
+    mbar_init(&bar_a, 4);                 // A rows written, one arrival per warp
+    mbar_init(&bar_d, 1);                 // products complete
+    for (int i = 0; i < NST; ++i) { mbar_init(&bar_full[i], C::NPROD / 32); mbar_init(&bar_free[i], 1); }
     asm volatile("fence.mbarrier_init.release.cluster;");
     abort_flag = 0;
   }
@@ -158,142 +231,197 @@ __global__ void __launch_bounds__(128) sample_tc_kernel(SampleArgs a) {
   __syncthreads();
   fence_after();
   const uint32_t tbase = tslot;
-  const uint32_t tlane = (uint32_t)(warp * 32) << 16;
-  uint32_t phase = 0;
 
-  // issue the 3xTF32 products for y = 0, 1 into TMEM columns [y*CHI, y*CHI + CHI)
-  auto issue = [&](const float* A0h, const float* A0l, const float* A1h, const float* A1l, const float* Bst) {
-    if (tid == 0) {
-      fence_after();
-#pragma unroll
-      for (int y = 0; y < 2; ++y) {
-        const float* Ah = y ? A1h : A0h;
-        const float* Al = y ? A1l : A0l;
-        const float* Bh = Bst + (y * 2 + 0) * BOP;
-        const float* Bl = Bst + (y * 2 + 1) * BOP;
-        const uint32_t d = tbase + (uint32_t)(y * CHI);
-        int first = 1;
-#pragma unroll
-        for (int term = 0; term < 3; ++term) {
-          const float* A = term == 2 ? Al : Ah;
-          const float* B = term == 1 ? Bl : Bh;
-#pragma unroll
-          for (int kk = 0; kk < KSTEPS; ++kk) {
-            mma_tf32(d, kmajor_desc(su32(A) + 256u * kk, SBO), kmajor_desc(su32(B) + 256u * kk, SBO), IDESC,
-                     first ? 0u : 1u);
-            first = 0;
-          }
-        }
-      }
-      mma_commit(&mbar);
+  // Bounded wait; on a timeout, or when another thread met one, every role leaves its loops and
+  // meets the others at the end.
+  auto wait_or_abort = [&](uint64_t* bar, uint32_t parity) -> bool {
+    for (int it = 0; it < (1 << 20); ++it) {
+      if (try_parity(bar, parity)) return true;
+      if (abort_flag) return false;
     }
-  };
-  // Wait for the products and load them.  On a timeout the thread records it, zeroes its
-  // values and carries on to the barrier that ends the site, where every thread sees the
-  // abort flag and leaves together.
-  auto finish = [&](float* v0, float* v1) -> bool {
-    const bool ok = wait_parity(&mbar, phase);
-    phase ^= 1u;
-    if (!ok) {
-      set_status(a.status, ST_TIMEOUT);
-      abort_flag = 1;
-#pragma unroll
-      for (int j = 0; j < CHI; ++j) { v0[j] = 0.0f; v1[j] = 0.0f; }
-      return false;
-    }
-    fence_after();
-    TmemLd<CHI>::ld(tbase + tlane + 0, v0);
-    TmemLd<CHI>::ld(tbase + tlane + CHI, v1);
-    tmem_wait_ld();
-    return true;
-  };
-  // convert prefetched tile values into a B stage (right: row al / K be; left: row be / K al)
-  auto convert = [&](const float* pre, float* Bst, bool left) {
-#pragma unroll
-    for (int i = 0; i < PRE; ++i) {
-      const int e = tid + M * i;                      // destination index over [y][d]
-      const int y = e / BOP, d = e % BOP;
-      const float x = pre[i];
-      const float h = tf32_rna(x), l = tf32_rna(x - h);
-      Bst[(y * 2 + 0) * BOP + d] = h;
-      Bst[(y * 2 + 1) * BOP + d] = l;
-    }
-    (void)left;
-  };
-  // source index (into the cached tile) of destination e for the right / left layouts
-  auto src_index = [&](int e, bool left) -> int {
-    const int y = e / BOP, d = e % BOP;
-    const int g = d / (8 * CHI), rem = d % (8 * CHI);
-    const int kg = rem / 32, rr = (rem % 32) / 4, kq = rem % 4;
-    const int row = 8 * g + rr, k = 4 * kg + kq;
-    return left ? (y * BOP + k * CHI + row) : (y * BOP + row * CHI + k);
-  };
-  auto prefetch = [&](const float* tile, float* pre, bool left) {
-#pragma unroll
-    for (int i = 0; i < PRE; ++i) pre[i] = __ldg(tile + src_index(tid + M * i, left));
+    set_status(a.status, ST_TIMEOUT);
+    abort_flag = 1;
+    return false;
   };
 
   const int tiles_per_real = (a.n_items + M - 1) / M;
   const int64_t total = (int64_t)tiles_per_real * a.n_real;
-  float* work = reinterpret_cast<float*>(a.work) + (size_t)blockIdx.x * L * 2 * M * CHI;
+  // Products per row: the right sweep's sites L-1 .. 1 (site 0's has no reader), then the left
+  // sweep's 0 .. L-1.
 
-  for (int64_t tileid = blockIdx.x; tileid < total; tileid += gridDim.x) {
-    const int real = (int)(tileid / tiles_per_real);
-    const int k = (int)(tileid % tiles_per_real) * M + tid;
-    const bool valid = k < a.n_items;
-    const int64_t item = (int64_t)real * a.n_items + k;
-    const int chain = a.forced ? 0 : (a.chain_of ? a.chain_of[real] : k / a.n);
-    const uint32_t step = (uint32_t)(a.step0 + (uint64_t)(a.forced ? 0 : k % a.n));
-    const uint64_t seed = a.seeds[real];
-    const double betad = a.beta[real];
-    const float eb = (float)exp(betad), ebm = (float)exp(-betad);
-    const int8_t* J = a.J + (size_t)real * 2 * L * (L - 1);
-    const float* envr = reinterpret_cast<const float*>(a.env) + (size_t)real * L * L * TILE;
-    const int8_t* forced = (a.forced && valid) ? a.forced + (size_t)item * N : nullptr;
-    const int8_t* hf = a.hfield ? a.hfield + (size_t)real * N : nullptr;
-    double logq = 0.0;
-    int energy = 0, magnet = 0;
-    long long nclamp = 0;
-    uint32_t gword = 0;
-
-    for (int r = 0; r < L; ++r) {
-      __syncthreads();
-      for (int c = tid; c < L - 1; c += M) jh_s[c] = J[(size_t)r * (L - 1) + c];
-      if (r > 0)
-        for (int c = tid; c < L; c += M) jv_s[c] = J[(size_t)L * (L - 1) + (size_t)(r - 1) * L + c];
-      const float* erow = envr + (size_t)r * L * TILE;
-      float pre[PRE];
-
-      // ---------------- right sweep ----------------
-      float R0[CHI], R1[CHI];
+  if (warp >= 5) {
+    // ---------------- tile warps ----------------
+    constexpr int UNITS = TILE / 4;                   // 16-byte chunks of a tile
+    constexpr int RS = CHI + 4;                       // row stride of a raw tile: the reads are conflict-free
+    const int ptid = tid - 160;
+    int64_t lt = blockIdx.x;                          // next tile to copy
+    int lr = 0, li = 0, lb = 0;
+    auto copy_next = [&]() {
+      if (lt < total) {
+        const int c = li < L - 1 ? L - 1 - li : li - (L - 1);
+        const float* tile = reinterpret_cast<const float*>(a.env) + (((size_t)(lt / tiles_per_real) * L + lr) * L + c) * TILE;
+        float* dst = Rawbuf + lb * C::RAWTILE;
+#pragma unroll 1
+        for (int u = ptid; u < UNITS; u += C::NPROD) {
+          const uint32_t d = su32(dst + (u / (CHI / 4)) * RS + 4 * (u % (CHI / 4)));
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(tile + 4 * u) : "memory");
+        }
+        lb = lb + 1 == raw_tiles ? 0 : lb + 1;
+        if (++li == 2 * L - 1) { li = 0; if (++lr == L) { lr = 0; lt += gridDim.x; } }
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    for (int d = 0; d < raw_tiles - 1; ++d) copy_next();
+    const int64_t mine = blockIdx.x < total ? (total - 1 - blockIdx.x) / gridDim.x + 1 : 0;
+    const int64_t operands = mine * L * (2 * L - 1);
+    int i = 0, rb = 0, st = 0;
+    uint32_t round = 0;                               // times the stages have been filled
+    for (int64_t n = 0; n < operands; ++n) {
+      // this tile's copy has arrived and the stage is free, for every tile warp; all are done with
+      // the raw tile before this one, whose buffer takes the next copy
+      if (raw_tiles > 2) asm volatile("cp.async.wait_group 1;" ::: "memory");
+      else asm volatile("cp.async.wait_group 0;" ::: "memory");
+      const bool ok = round == 0 || wait_or_abort(&bar_free[st], (round - 1) & 1u);
+      if (any_of<C::NPROD>(1, !ok)) break;            // all of them leave, or none
+      copy_next();
+      const bool left = i >= L - 1;
+      const float* src = Rawbuf + rb * C::RAWTILE;
+      float* stage = Bbuf + st * C::STAGE;
+#pragma unroll 1
+      for (int u = ptid; u < UNITS; u += C::NPROD) {
+        // right: four be of row al; left: four al of row be
+        const int y = u / (UNITS / 2), e = u % (UNITS / 2);
+        const float* p = src + y * CHI * RS;
+        int row, kg;
+        float x[4];
+        if (left) {
+          row = e % CHI; kg = e / CHI;
 #pragma unroll
-      for (int j = 0; j < CHI; ++j) { R0[j] = (j == 0) ? 1.0f : 0.0f; R1[j] = R0[j]; }
-      put_row_split<CHI>(Abuf + 0 * AOP, Abuf + 1 * AOP, tid, R0);
-      put_row_split<CHI>(Abuf + 2 * AOP, Abuf + 3 * AOP, tid, R1);
-      prefetch(erow + (size_t)(L - 1) * TILE, pre, false);
-      convert(pre, Bbuf, false);
-      if (L > 1) prefetch(erow + (size_t)(L - 2) * TILE, pre, false);
+          for (int t = 0; t < 4; ++t) x[t] = p[(4 * kg + t) * RS + row];
+        } else {
+          row = (e / (2 * CHI)) * 8 + (e & 7); kg = (e >> 3) % (CHI / 4);
+          const float4 v = *reinterpret_cast<const float4*>(p + row * RS + 4 * kg);
+          x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+        }
+        float h[4], l[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) { h[t] = tf32_rna(x[t]); l[t] = tf32_rna(x[t] - h[t]); }
+        float* d = stage + y * BOP + koff<CHI>(row, 4 * kg);
+        *reinterpret_cast<float4*>(d) = make_float4(h[0], h[1], h[2], h[3]);
+        *reinterpret_cast<float4*>(d + 2 * BOP) = make_float4(l[0], l[1], l[2], l[3]);
+      }
       fence_async_smem();
-      fence_before();
-      __syncthreads();
-      for (int ci = 0; ci < L; ++ci) {
-        const int c = L - 1 - ci, st = ci & 1;
-        issue(Abuf + 0 * AOP, Abuf + 1 * AOP, Abuf + 2 * AOP, Abuf + 3 * AOP, Bbuf + st * 4 * BOP);
-        if (c > 0) {
-          convert(pre, Bbuf + (st ^ 1) * 4 * BOP, false);
-          if (c > 1) prefetch(erow + (size_t)(c - 2) * TILE, pre, false);
-          fence_async_smem();
-        }
-        float v0[CHI], v1[CHI];
-        finish(v0, v1);
-        // R_{c+1}(y) -> workspace (read back by the left sweep at site c)
-        float* wsl = work + ((size_t)(c * 2) * M + tid) * CHI;
+      __syncwarp();
+      if ((tid & 31) == 0) mbar_arrive(&bar_full[st]);
+      if (++i == 2 * L - 1) i = 0;
+      rb = rb + 1 == raw_tiles ? 0 : rb + 1;
+      if (++st == NST) { st = 0; ++round; }
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+  } else if (warp == 4) {
+    // ---------------- MMA warp ----------------
+    // the whole warp runs the loop, one lane is elected at each issue: descriptors and addresses
+    // stay in uniform registers
+    uint32_t n = 0, round = 0;
+    int st = 0;
+    bool run = true;
+    const uint32_t ta = tbase + 2 * CHI;
+    constexpr uint64_t LO = (uint64_t)(2 * BOP * 4) >> 4, Y1 = (uint64_t)(BOP * 4) >> 4, KK = 256u >> 4;
+    const uint64_t b0 = kmajor_desc(su32(Bbuf), SBO);
+    for (int64_t tileid = blockIdx.x; run && tileid < total; tileid += gridDim.x)
+      for (int r = 0; run && r < L; ++r)
+        for (int i = 0; i < 2 * L - 1; ++i) {
+          const bool ok = wait_or_abort(&bar_full[st], round & 1u) && wait_or_abort(&bar_a, n & 1u);
+          if (!__all_sync(0xffffffffu, ok)) { run = false; break; }
+          fence_after();
+          const uint64_t bh = b0 + (uint64_t)st * ((C::STAGE * 4) >> 4);
+          if (elect_one()) {
+            // hi.hi + hi.lo + lo.hi, each over K in steps of 8
+            if (i < L - 1) {
 #pragma unroll
-        for (int j = 0; j < CHI; j += 4) {
-          *reinterpret_cast<float4*>(wsl + j) = make_float4(R0[j], R0[j + 1], R0[j + 2], R0[j + 3]);
-          *reinterpret_cast<float4*>(wsl + (size_t)M * CHI + j) = make_float4(R1[j], R1[j + 1], R1[j + 2], R1[j + 3]);
+              for (int y = 0; y < 2; ++y)
+#pragma unroll
+                for (int term = 0; term < 3; ++term)
+#pragma unroll
+                  for (int kk = 0; kk < CHI / 8; ++kk)
+                    mma_tf32(tbase + y * CHI, ta + (2 * y + (term == 2 ? 1 : 0)) * CHI + 8 * kk,
+                             bh + (term == 1 ? LO : 0) + y * Y1 + kk * KK, idesc_tf32<CHI>(), (term | kk) ? 1u : 0u);
+            } else {
+#pragma unroll
+              for (int term = 0; term < 3; ++term)
+#pragma unroll
+                for (int kk = 0; kk < CHI / 8; ++kk)
+                  mma_tf32(tbase, ta + (term == 2 ? CHI : 0) + 8 * kk, bh + (term == 1 ? LO : 0) + kk * KK,
+                           idesc_tf32<2 * CHI>(), (term | kk) ? 1u : 0u);
+            }
+            mma_commit(&bar_d);
+            mma_commit(&bar_free[st]);
+          }
+          __syncwarp();
+          ++n;
+          if (++st == NST) { st = 0; ++round; }
         }
-        if (c > 0) {
+    if (!run && n > 0) wait_parity(&bar_d, (n - 1) & 1);       // products in flight end before the memory is freed
+    __syncwarp();
+  } else {
+    // ---------------- proposal warps ----------------
+    const uint32_t tlane = (uint32_t)(warp * 32) << 16;
+    const uint32_t td = tbase + tlane, ta = td + 2 * CHI;
+    const int lane = tid & 31;
+    int8_t* jh_s = jrow + warp * 2 * LP;
+    int8_t* jv_s = jh_s + LP;
+    uint32_t n = 0;                                   // products waited for
+    bool run = true;
+    // the products are complete (warp-uniform: the TMEM accesses need the whole warp)
+    auto products = [&]() -> bool {
+      const bool ok = __all_sync(0xffffffffu, wait_or_abort(&bar_d, n & 1));
+      ++n;
+      fence_after();
+      return ok;
+    };
+    auto a_ready = [&]() {                            // this warp's A rows are written
+      tmem_wait_st();
+      fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&bar_a);
+    };
+    // R_{c+1}(y) per site and proposal, [site][y][j / 4][proposal][4]: 16-byte accesses that are
+    // contiguous over the lanes
+    float* work = reinterpret_cast<float*>(a.work) + (size_t)blockIdx.x * L * 2 * M * CHI + 4 * tid;
+    float* rws = Rws + 4 * tid;                       // one site's, in shared memory
+
+    for (int64_t tileid = blockIdx.x; run && tileid < total; tileid += gridDim.x) {
+      const int real = (int)(tileid / tiles_per_real);
+      const int k = (int)(tileid % tiles_per_real) * M + tid;
+      const bool valid = k < a.n_items;
+      const int64_t item = (int64_t)real * a.n_items + k;
+      const int chain = a.forced ? 0 : (a.chain_of ? a.chain_of[real] : k / a.n);
+      const uint32_t step = (uint32_t)(a.step0 + (uint64_t)(a.forced ? 0 : k % a.n));
+      const uint64_t seed = a.seeds[real];
+      const double betad = a.beta[real];
+      const float eb = (float)exp(betad), ebm = (float)exp(-betad);
+      const int8_t* J = a.J + (size_t)real * 2 * L * (L - 1);
+      const int8_t* forced = (a.forced && valid) ? a.forced + (size_t)item * N : nullptr;
+      const int8_t* hf = a.hfield ? a.hfield + (size_t)real * N : nullptr;
+      double logq = 0.0;
+      int energy = 0, magnet = 0;
+      long long nclamp = 0;
+      uint32_t gword = 0;
+
+      for (int r = 0; r < L; ++r) {
+        // the couplings of this row, a copy per warp: no barrier between the warps
+        __syncwarp();
+        for (int c = lane; c < L - 1; c += 32) jh_s[c] = J[(size_t)r * (L - 1) + c];
+        if (r > 0)
+          for (int c = lane; c < L; c += 32) jv_s[c] = J[(size_t)L * (L - 1) + (size_t)(r - 1) * L + c];
+        __syncwarp();
+
+        // ---------------- right sweep ----------------
+        put_e0<CHI>(ta);
+        put_e0<CHI>(ta + 2 * CHI);
+        a_ready();
+        for (int c = L - 1; c > 0; --c) {
+          // R_c(y') = sum_y exp(beta Jh s_y' s_y) exp(h_c s_y) v_y
           const int jh = jh_s[c - 1];
           float f0 = 1.0f, f1 = 1.0f;
           if (r > 0) {
@@ -303,189 +431,252 @@ __global__ void __launch_bounds__(128) sample_tc_kernel(SampleArgs a) {
           }
           if (hf) { const int kh = hf[(size_t)r * L + c]; if (kh) { f0 *= expf((float)(betad * kh)); f1 *= expf((float)(-betad * kh)); } }
           const float same = jh > 0 ? eb : ebm, diff = jh > 0 ? ebm : eb;
-          float mx = 0.0f;
+          const float s0 = same * f0, s1 = same * f1, d0 = diff * f0, d1 = diff * f1;
+          if (!products()) { run = false; break; }
+          // eight columns at a time, in loops that are not unrolled: a straight-line body is
+          // fetched anew for every site (see the head of the kernel)
+          auto combine = [&](int j, float* n0, float* n1) {
+            float v0[8], v1[8];
+            tmem_ld8(td + j, v0);
+            tmem_ld8(td + CHI + j, v1);
+            tmem_wait_ld();
 #pragma unroll
-          for (int j = 0; j < CHI; ++j) {
-            const float n0 = same * f0 * v0[j] + diff * f1 * v1[j];
-            const float n1 = diff * f0 * v0[j] + same * f1 * v1[j];
-            R0[j] = n0; R1[j] = n1;
-            mx = fmaxf(mx, fmaxf(fabsf(n0), fabsf(n1)));
+            for (int t = 0; t < 8; ++t) {
+              n0[t] = fmaf(s0, v0[t], __fmul_rn(d1, v1[t]));
+              n1[t] = fmaf(d0, v0[t], __fmul_rn(s1, v1[t]));
+            }
+          };
+          float mx0 = 0.0f, mx1 = 0.0f;
+#pragma unroll 1
+          for (int j = 0; j < CHI; j += 8) {
+            float n0[8], n1[8];
+            combine(j, n0, n1);
+#pragma unroll
+            for (int t = 0; t < 8; ++t) { mx0 = max_nan(mx0, fabsf(n0[t])); mx1 = max_nan(mx1, fabsf(n1[t])); }
+          }
+          float mx = max_nan(mx0, mx1);
+          if (__any_sync(0xffffffffu, isnan(mx))) {      // a NaN takes no part in the maximum
+            mx = 0.0f;
+#pragma unroll 1
+            for (int j = 0; j < CHI; j += 8) {
+              float n0[8], n1[8];
+              combine(j, n0, n1);
+#pragma unroll
+              for (int t = 0; t < 8; ++t) mx = fmaxf(mx, fmaxf(fabsf(n0[t]), fabsf(n1[t])));
+            }
           }
           const float inv = mx > 0.0f ? 1.0f / mx : 1.0f;
+          const bool fin = __all_sync(0xffffffffu, !isnan(max_nan(mx0, mx1)) && isfinite(mx) && isfinite(inv));
+          // read back by the left sweep at c - 1 (the last one at once, so it stays on the chip)
+          float* wsl = c > 1 ? work + (size_t)((c - 1) * 2) * M * CHI : rws;
+#pragma unroll 1
+          for (int j = 0; j < CHI; j += 8) {
+            float n0[8], n1[8];
+            combine(j, n0, n1);
 #pragma unroll
-          for (int j = 0; j < CHI; ++j) { R0[j] *= inv; R1[j] *= inv; }
-          put_row_split<CHI>(Abuf + 0 * AOP, Abuf + 1 * AOP, tid, R0);
-          put_row_split<CHI>(Abuf + 2 * AOP, Abuf + 3 * AOP, tid, R1);
-          fence_async_smem();
+            for (int t = 0; t < 8; ++t) { n0[t] *= inv; n1[t] *= inv; }
+#pragma unroll
+            for (int t = 0; t < 8; t += 4) {
+              *reinterpret_cast<float4*>(wsl + (j + t) * M) = make_float4(n0[t], n0[t + 1], n0[t + 2], n0[t + 3]);
+              *reinterpret_cast<float4*>(wsl + (CHI + j + t) * M) = make_float4(n1[t], n1[t + 1], n1[t + 2], n1[t + 3]);
+            }
+            put8_split<CHI>(ta + j, n0, fin);
+            put8_split<CHI>(ta + 2 * CHI + j, n1, fin);
+          }
+          if (c > 1) a_ready();
         }
-        fence_before();
-        __syncthreads();
-        if (abort_flag) break;
-      }
-      if (abort_flag) break;
+        if (!run) break;
 
-      // ---------------- left sweep ----------------
-      float ell[CHI];
+        __threadfence();              // the copies below read what this thread has stored
+        // ---------------- left sweep ----------------
+        put_e0<CHI>(ta);
+        a_ready();
+        int sprev = 0;
+        float rsum = 0.0f, rcomp = 0.0f;
+        uint32_t rword = 0;
+        for (int c = 0; c < L; ++c) {
+          // what does not depend on the products: the fields, the random number
+          float f0 = 1.0f, f1 = 1.0f;
+          int sp = 0;
+          if (r > 0) {
+            sp = ((prow[(c >> 5) * M + tid] >> (c & 31)) & 1u) ? -1 : 1;
+            const int sg = jv_s[c] * sp;
+            f0 = sg > 0 ? eb : ebm; f1 = sg > 0 ? ebm : eb;
+          }
+          if (c > 0) { const int sg = jh_s[c - 1] * sprev; f0 *= sg > 0 ? eb : ebm; f1 *= sg > 0 ? ebm : eb; }
+          if (hf) { const int kh = hf[(size_t)r * L + c]; if (kh) { f0 *= expf((float)(betad * kh)); f1 *= expf((float)(-betad * kh)); } }
+          uint64_t m53 = 0;
+          int sforced = 0;
+          if (forced) {
+            sforced = forced[(size_t)r * L + c];
+          } else {
+            const Philox4 o = philox4x32_10((uint32_t)(r * L + c), step, (uint32_t)chain, PURPOSE_SPIN,
+                                            (uint32_t)seed, (uint32_t)(seed >> 32));
+            m53 = ((uint64_t)(o.x0 >> 5) << 26) | (uint64_t)(o.x1 >> 6);
+          }
+          if (!products()) { run = false; break; }
+          asm volatile("cp.async.wait_group 0;" ::: "memory");
+          float d0 = 0.0f, d1 = 0.0f;
+#pragma unroll 1
+          for (int j = 0; j < CHI; j += 8) {
+            float u0[8], u1[8], r0[8], r1[8];
+            tmem_ld8(td + j, u0);
+            tmem_ld8(td + CHI + j, u1);
 #pragma unroll
-      for (int j = 0; j < CHI; ++j) ell[j] = (j == 0) ? 1.0f : 0.0f;
-      put_row_split<CHI>(Abuf + 0 * AOP, Abuf + 1 * AOP, tid, ell);
-      prefetch(erow, pre, true);
-      convert(pre, Bbuf, true);
-      if (L > 1) prefetch(erow + (size_t)1 * TILE, pre, true);
-      fence_async_smem();
-      fence_before();
-      __syncthreads();
-      int sprev = 0;
-      float rsum = 0.0f, rcomp = 0.0f;
-      uint32_t rword = 0;
-      for (int c = 0; c < L; ++c) {
-        const int st = c & 1;
-        issue(Abuf + 0 * AOP, Abuf + 1 * AOP, Abuf + 0 * AOP, Abuf + 1 * AOP, Bbuf + st * 4 * BOP);
-        if (c + 1 < L) {
-          convert(pre, Bbuf + (st ^ 1) * 4 * BOP, true);
-          if (c + 2 < L) prefetch(erow + (size_t)(c + 2) * TILE, pre, true);
-          fence_async_smem();
-        }
-        float Rw0[CHI], Rw1[CHI];
-        const float* wsl = work + ((size_t)(c * 2) * M + tid) * CHI;
+            for (int t = 0; t < 8; t += 4) {
+              *reinterpret_cast<float4*>(r0 + t) = *reinterpret_cast<const float4*>(rws + (j + t) * M);
+              *reinterpret_cast<float4*>(r1 + t) = *reinterpret_cast<const float4*>(rws + (CHI + j + t) * M);
+            }
+            tmem_wait_ld();
 #pragma unroll
-        for (int j = 0; j < CHI; j += 4) {
-          const float4 p0 = *reinterpret_cast<const float4*>(wsl + j);
-          const float4 p1 = *reinterpret_cast<const float4*>(wsl + (size_t)M * CHI + j);
-          Rw0[j] = p0.x; Rw0[j + 1] = p0.y; Rw0[j + 2] = p0.z; Rw0[j + 3] = p0.w;
-          Rw1[j] = p1.x; Rw1[j + 1] = p1.y; Rw1[j + 2] = p1.z; Rw1[j + 3] = p1.w;
-        }
-        float u0[CHI], u1[CHI];
-        finish(u0, u1);
-        float d0 = 0.0f, d1 = 0.0f;
+            for (int t = 0; t < 8; ++t) { d0 = fmaf(u0[t], r0[t], d0); d1 = fmaf(u1[t], r1[t], d1); }
+          }
+          // the next site's right vectors: a copy in flight while this site is finished
+          if (c + 2 < L) {
+            const float* wsl = work + (size_t)((c + 1) * 2) * M * CHI;
+#pragma unroll 4
+            for (int j = 0; j < 2 * CHI; j += 4)
+              asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(su32(rws + j * M)), "l"(wsl + j * M) : "memory");
+            asm volatile("cp.async.commit_group;" ::: "memory");
+          } else if (c + 1 < L) {
+#pragma unroll 4
+            for (int j = 0; j < 2 * CHI; j += 4)
+              *reinterpret_cast<float4*>(rws + j * M) = make_float4(j % CHI == 0 ? 1.0f : 0.0f, 0.0f, 0.0f, 0.0f);
+          }
+          float w0 = f0 * d0, w1 = f1 * d1;
+          if (w0 < 0.0f) { w0 = 0.0f; ++nclamp; }
+          if (w1 < 0.0f) { w1 = 0.0f; ++nclamp; }
+          const float tot = w0 + w1;
+          const bool bad = !(tot > 0.0f) || !isfinite(tot);
+          // A doubly clamped or non-finite site flags the realization; the spin is still drawn from
+          // the q = 1/2 that is logged, so that log q stays the probability of the proposal.
+          const float qp = bad ? 0.5f : w0 / tot;
+          const int s = forced ? sforced : (bad ? ((m53 < (1ull << 52)) ? 1 : -1) : (draw_below(m53, qp) ? 1 : -1));
+          // l <- u_s, normalised
+          if (c < L - 1) {
+            auto chosen = [&](int j, float* x) {
+              float u1[8];
+              tmem_ld8(td + j, x);
+              tmem_ld8(td + CHI + j, u1);
+              tmem_wait_ld();
 #pragma unroll
-        for (int j = 0; j < CHI; ++j) { d0 += u0[j] * Rw0[j]; d1 += u1[j] * Rw1[j]; }
-        float f0 = 1.0f, f1 = 1.0f;
-        int sp = 0;
-        if (r > 0) {
-          sp = ((prow[(c >> 5) * M + tid] >> (c & 31)) & 1u) ? -1 : 1;
-          const int sg = jv_s[c] * sp;
-          f0 = sg > 0 ? eb : ebm; f1 = sg > 0 ? ebm : eb;
-        }
-        if (c > 0) { const int sg = jh_s[c - 1] * sprev; f0 *= sg > 0 ? eb : ebm; f1 *= sg > 0 ? ebm : eb; }
-        if (hf) { const int kh = hf[(size_t)r * L + c]; if (kh) { f0 *= expf((float)(betad * kh)); f1 *= expf((float)(-betad * kh)); } }
-        float w0 = f0 * d0, w1 = f1 * d1;
-        if (w0 < 0.0f) { w0 = 0.0f; ++nclamp; }
-        if (w1 < 0.0f) { w1 = 0.0f; ++nclamp; }
-        const float tot = w0 + w1;
-        int s;
-        float qp = 0.5f, lqs;
-        if (!(tot > 0.0f) || !isfinite(tot)) {
-          if (valid) {
+              for (int t = 0; t < 8; ++t) x[t] = s == 1 ? x[t] : u1[t];
+            };
+            __syncwarp();
+            float mx0 = 0.0f, mx1 = 0.0f;
+#pragma unroll 1
+            for (int j = 0; j < CHI; j += 8) {
+              float x[8];
+              chosen(j, x);
+#pragma unroll
+              for (int t = 0; t < 8; t += 2) { mx0 = max_nan(mx0, fabsf(x[t])); mx1 = max_nan(mx1, fabsf(x[t + 1])); }
+            }
+            float mx = max_nan(mx0, mx1);
+            if (__any_sync(0xffffffffu, isnan(mx))) {
+              mx = 0.0f;
+#pragma unroll 1
+              for (int j = 0; j < CHI; j += 8) {
+                float x[8];
+                chosen(j, x);
+#pragma unroll
+                for (int t = 0; t < 8; ++t) mx = fmaxf(mx, fabsf(x[t]));
+              }
+            }
+            const float inv = mx > 0.0f ? 1.0f / mx : 1.0f;
+            const bool fin = __all_sync(0xffffffffu, !isnan(max_nan(mx0, mx1)) && isfinite(mx) && isfinite(inv));
+#pragma unroll 1
+            for (int j = 0; j < CHI; j += 8) {
+              float x[8];
+              chosen(j, x);
+#pragma unroll
+              for (int t = 0; t < 8; ++t) x[t] *= inv;
+              put8_split<CHI>(ta + j, x, fin);
+            }
+            a_ready();
+          }
+          // what the next product does not wait for: log q, the output, the energy
+          float lqs = -0.6931471805599453f;
+          if (!bad) {
+            const float qm = w1 / tot;
+            const float qs = s == 1 ? qp : qm, qo = s == 1 ? qm : qp;
+            lqs = qs > 0.5f ? log1pf(-qo) : logf(qs);
+          } else if (valid) {
             set_status(a.status, ST_NUMERIC);
             if (a.real_status) set_status(a.real_status + real, ST_NUMERIC);
           }
-          // the realization is flagged; the spin is still drawn from the q = 1/2 it logs,
-          // so that log q stays the probability the proposal was drawn with
-          if (forced) {
-            s = forced[(size_t)r * L + c];
-          } else {
-            const Philox4 o = philox4x32_10((uint32_t)(r * L + c), step, (uint32_t)chain, PURPOSE_SPIN,
-                                            (uint32_t)seed, (uint32_t)(seed >> 32));
-            s = ((o.x0 >> 5) < (1u << 26)) ? 1 : -1;      // m53 < 2^52
+          { const float yk = lqs - rcomp; const float tk = rsum + yk; rcomp = (tk - rsum) - yk; rsum = tk; }
+          if (a.qplus && valid) a.qplus[(size_t)item * N + (size_t)r * L + c] = (double)qp;
+          if (c > 0) energy -= jh_s[c - 1] * sprev * s;
+          if (r > 0) energy -= jv_s[c] * sp * s;
+          magnet += s;
+          sprev = s;
+          if (s < 0) rword |= 1u << (c & 31);
+          // the previous row's word has been read to its end
+          if ((c & 31) == 31 || c == L - 1) { prow[(c >> 5) * M + tid] = rword; rword = 0; }
+          const int site = r * L + c;
+          if (s < 0) gword |= 1u << (site & 31);
+          if ((site & 31) == 31 || site == N - 1) {
+            if (valid && a.spins_packed) a.spins_packed[(size_t)item * a.words + (site >> 5)] = gword;
+            gword = 0;
           }
-          lqs = -0.6931471805599453f;
-        } else {
-          qp = w0 / tot;
-          const float qm = w1 / tot;
-          if (forced) {
-            s = forced[(size_t)r * L + c];
-          } else {
-            const Philox4 o = philox4x32_10((uint32_t)(r * L + c), step, (uint32_t)chain, PURPOSE_SPIN,
-                                            (uint32_t)seed, (uint32_t)(seed >> 32));
-            const uint64_t m53 = ((uint64_t)(o.x0 >> 5) << 26) | (uint64_t)(o.x1 >> 6);
-            // u < q(+) exactly: m < ceil(q 2^53) (q a float in (0, 1))
-            bool below = false;
-            if (qp >= 1.0f) below = true;
-            else if (qp > 0.0f) {
-              const uint32_t bits = __float_as_uint(qp);
-              const int ex = (int)((bits >> 23) & 0xffu);
-              const uint64_t mant = (ex == 0) ? (uint64_t)(bits & 0x7fffffu) : (uint64_t)((bits & 0x7fffffu) | 0x800000u);
-              const int sh = (ex == 0 ? 1 : ex) - 150 + 53;
-              uint64_t C;
-              if (sh >= 0) C = mant << sh;
-              else { const int kq = -sh; C = (kq >= 64) ? 1ull : ((mant + ((1ull << kq) - 1ull)) >> kq); }
-              below = m53 < C;
-            }
-            s = below ? 1 : -1;
-          }
-          const float qs = s == 1 ? qp : qm, qo = s == 1 ? qm : qp;
-          lqs = qs > 0.5f ? log1pf(-qo) : logf(qs);
         }
-        { const float yk = lqs - rcomp; const float tk = rsum + yk; rcomp = (tk - rsum) - yk; rsum = tk; }
-        if (a.qplus && valid) a.qplus[(size_t)item * N + (size_t)r * L + c] = (double)qp;
-        // l <- u_s, normalised
-        float mx = 0.0f;
-#pragma unroll
-        for (int j = 0; j < CHI; ++j) { ell[j] = s == 1 ? u0[j] : u1[j]; mx = fmaxf(mx, fabsf(ell[j])); }
-        const float inv = mx > 0.0f ? 1.0f / mx : 1.0f;
-#pragma unroll
-        for (int j = 0; j < CHI; ++j) ell[j] *= inv;
-        put_row_split<CHI>(Abuf + 0 * AOP, Abuf + 1 * AOP, tid, ell);
-        fence_async_smem();
-        if (c > 0) energy -= jh_s[c - 1] * sprev * s;
-        if (r > 0) energy -= jv_s[c] * sp * s;
-        magnet += s;
-        sprev = s;
-        if (s < 0) rword |= 1u << (c & 31);
-        if ((c & 31) == 31 || c == L - 1) { crow[(c >> 5) * M + tid] = rword; rword = 0; }
-        const int site = r * L + c;
-        if (s < 0) gword |= 1u << (site & 31);
-        if ((site & 31) == 31 || site == N - 1) {
-          if (valid && a.spins_packed) a.spins_packed[(size_t)item * a.words + (site >> 5)] = gword;
-          gword = 0;
-        }
-        fence_before();
-        __syncthreads();
-        if (abort_flag) break;
+        if (!run) break;
+        logq += (double)rsum;
       }
-      if (abort_flag) break;
-      logq += (double)rsum;
-      for (int w = 0; w < words_row; ++w) prow[w * M + tid] = crow[w * M + tid];
+      if (valid && run) {
+        if (a.logq) a.logq[item] = logq;
+        if (a.energy) a.energy[item] = energy;
+        if (a.magnet) a.magnet[item] = magnet;
+        if (a.clamps && nclamp) atomicAdd(reinterpret_cast<unsigned long long*>(a.clamps + real), (unsigned long long)nclamp);
+      }
     }
-    if (valid && !abort_flag) {
-      if (a.logq) a.logq[item] = logq;
-      if (a.energy) a.energy[item] = energy;
-      if (a.magnet) a.magnet[item] = magnet;
-      if (a.clamps && nclamp) atomicAdd(reinterpret_cast<unsigned long long*>(a.clamps + real), (unsigned long long)nclamp);
-    }
-    if (abort_flag) break;
   }
   fence_before();
   __syncthreads();
-  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tbase), "r"(TCOLS));
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tbase), "r"(C::TCOLS));
 }
 
 template <int CHI>
-static size_t sample_tc_smem(int L) {
+static size_t sample_tc_smem(int L, int raw_tiles) {
+  using C = tc::Cfg<CHI>;
   const int words_row = (L + 31) / 32;
-  return (size_t)(4 * tc::M * CHI + 8 * CHI * CHI) * sizeof(float) + (size_t)2 * ((L + 15) & ~15) +
-         (size_t)2 * words_row * tc::M * sizeof(uint32_t) + 64;
+  return (size_t)(C::NST * C::STAGE + raw_tiles * C::RAWTILE + 2 * CHI * tc::M) * sizeof(float) +
+         (size_t)8 * ((L + 15) & ~15) + (size_t)words_row * tc::M * sizeof(uint32_t) + 64;
 }
 
-int sample_tc_grid(int n_items, int n_real, int num_sms) {
+static int per_sm(int CHI) { return CHI <= 16 ? tc::Cfg<16>::PER_SM : tc::Cfg<32>::PER_SM; }
+
+static int sample_tc_grid(int n_items, int n_real, int CHI, int num_sms) {
   const int64_t tiles = (int64_t)((n_items + tc::M - 1) / tc::M) * n_real;
-  int64_t grid = (int64_t)num_sms * 2;
+  int64_t grid = (int64_t)num_sms * per_sm(CHI);
   if (grid > tiles) grid = tiles;
   return grid < 1 ? 1 : (int)grid;
 }
 
 size_t sample_tc_work_bytes(int L, int CHI, int num_sms) {
-  return (size_t)num_sms * 2 * (size_t)L * 2 * tc::M * CHI * sizeof(float);
+  return (size_t)num_sms * per_sm(CHI) * (size_t)L * 2 * tc::M * CHI * sizeof(float);
 }
 
 template <int CHI>
 static cudaError_t launch_tc_t(const SampleArgs& a, int num_sms, cudaStream_t st) {
-  const size_t smem = sample_tc_smem<CHI>(a.L);
-  cudaError_t e = cudaFuncSetAttribute(sample_tc_kernel<CHI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  const int grid = sample_tc_grid(a.n_items, a.n_real, num_sms);
-  sample_tc_kernel<CHI><<<grid, tc::M, smem, st>>>(a);
+  // Three raw tiles in flight where PER_SM CTAs still fit on an SM (CHI = 32: L up to about 210), else
+  // two: at L = 256 a second CTA is worth more than the third tile.
+  int raw_tiles = 3, fit = 0;
+  size_t smem = 0;
+  for (;; --raw_tiles) {
+    smem = sample_tc_smem<CHI>(a.L, raw_tiles);
+    cudaError_t e = cudaFuncSetAttribute(sample_tc_kernel<CHI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess)
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, sample_tc_kernel<CHI>, tc::Cfg<CHI>::NT, smem);
+    if (e == cudaSuccess && fit >= tc::Cfg<CHI>::PER_SM) break;
+    if (raw_tiles == 2) {
+      if (e != cudaSuccess) return e;
+      break;
+    }
+    cudaGetLastError();
+  }
+  const int grid = sample_tc_grid(a.n_items, a.n_real, CHI, num_sms);
+  sample_tc_kernel<CHI><<<grid, tc::Cfg<CHI>::NT, smem, st>>>(a, raw_tiles);
   return cudaGetLastError();
 }
 
