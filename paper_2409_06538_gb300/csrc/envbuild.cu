@@ -1005,9 +1005,14 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
       __syncthreads();
       const int k = min(chi, min(dqr[c], n));
       if (tid < n) {
-        const T sj = sig[tid];
+        // a NaN ranks below every norm, so that the ranks are a permutation and all of sel is set
+        // whatever the columns hold (an overflowed realization is flagged when it is sampled)
+        const T sn = sig[tid], sj = sn >= T(0) ? sn : T(-1);
         int rank = 0;
-        for (int i = 0; i < n; ++i) { const T si = sig[i]; rank += (si > sj) || (si == sj && i < tid); }
+        for (int i = 0; i < n; ++i) {
+          const T st = sig[i], si = st >= T(0) ? st : T(-1);
+          rank += (si > sj) || (si == sj && i < tid);
+        }
         if (rank < k) sel[rank] = tid;
       }
       if (tid == 0) { knew[mir ? L - c : c] = k; knext_s = k; }
