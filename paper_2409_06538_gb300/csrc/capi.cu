@@ -199,9 +199,10 @@ CtxSizes ctx_sizes(int L, int n_real, int CHI, int precision, int n_chains, int 
   z.stats = 4 * sizeof(long long) * R;
   z.status = sizeof(unsigned);
   z.rstatus = sizeof(unsigned) * R;
-  z.work = tnmc::sample_work_bytes(L, CHI, precision, num_sms);
-  z.work_tc = (precision == TNMC_MIXED_TF32 && tnmc::sample_tc_supported(CHI))
-                  ? tnmc::sample_tc_work_bytes(L, CHI, num_sms) : 0;
+  // one workspace: that of the sampler which serves the context
+  const bool tc = precision == TNMC_MIXED_TF32 && tnmc::sample_tc_supported(CHI);
+  z.work = tc ? 0 : tnmc::sample_work_bytes(L, CHI, precision, num_sms);
+  z.work_tc = tc ? tnmc::sample_tc_work_bytes(L, CHI, num_sms) : 0;
   z.clamps = 8 * R;
   z.have_state = 4 * chains; z.cur_logq = 8 * chains; z.cur_energy = 4 * chains; z.cur_magnet = 4 * chains;
   z.cur_spins = 4 * chains * words;
@@ -319,7 +320,7 @@ tnmc_status tnmc_create(int L, int n_real, const int8_t* couplings, const double
   TRY(dalloc(c, &c->stats, z.stats));
   TRY(dalloc(c, &c->status, z.status));
   TRY(dalloc(c, &c->rstatus, z.rstatus));
-  TRY(dalloc(c, &c->work, z.work));
+  if (z.work) TRY(dalloc(c, &c->work, z.work));
   if (z.work_tc) TRY(dalloc(c, &c->work_tc, z.work_tc));
   TRY(dalloc(c, &c->clamps, z.clamps));
   const size_t chains = (size_t)n_real * c->n_chains;
@@ -472,6 +473,7 @@ static tnmc_status run_sample(tnmc_ctx* c, int n, uint64_t step0, const int8_t* 
   a.real_status = props ? c->rstatus : nullptr;
   a.hfield = c->hfield;
   a.chain_of = props ? c->chain_of : nullptr;
+  a.kdim = c->kdim;
   cudaError_t e;
   if (c->work_tc) {
     a.work = c->work_tc;

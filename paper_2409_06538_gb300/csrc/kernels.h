@@ -63,6 +63,7 @@ struct SampleArgs {
   unsigned* real_status;           // [real] per-realization status bits (nullable)
   const int8_t* hfield;            // [real][L][L] external fields in units of beta (nullable)
   const int* chain_of;             // [real] chain index of the draws' counters (nullable: item / n)
+  const int* kdim;                 // [real][L rows][L+1] bond dimensions of the environments
 };
 
 cudaError_t launch_sample(const SampleArgs& a, int precision, int CHI, int num_sms, cudaStream_t st);
