@@ -114,8 +114,8 @@ template <typename T> __device__ __forceinline__ T group8_sum(T v) {
   v += __shfl_xor_sync(0xffffffffu, v, 4);
   return v;
 }
-__device__ __forceinline__ void named_barrier(int id, int nthreads) {
-  asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(nthreads) : "memory");
+template <int ID> __device__ __forceinline__ void named_barrier(int nthreads) {
+  asm volatile("bar.sync %0, %1;\n" ::"n"(ID), "r"(nthreads) : "memory");
 }
 
 // 4-element shared-memory vectors (16 B for float, 2 x 16 B for double); callers keep the
@@ -145,13 +145,23 @@ __device__ __forceinline__ void prefetch_async(void* smem, const void* gmem, int
   cp_async_commit_env();
 }
 
-template <int CHI> struct EnvCfg {
+template <int CHI, bool kCrowd = false> struct EnvCfg {
   static constexpr int D = 2 * CHI;                 // MPO bond x MPS bond
-  // 8 lanes per Jacobi pair (8*CHI threads); CHI = 32 runs 256 threads so that three
-  // realizations fit on one SM in FP32 (80 registers, 72 KB of shared memory each)
-  // CHI = 64 runs 512 threads (64 Jacobi pairs) with one CTA per SM
-  static constexpr int NWARP = CHI > 32 ? 16 : (CHI < 4 ? 4 : (CHI > 8 ? 8 : CHI));
-  static constexpr int NT = 32 * NWARP;
+  // 8 CHI threads: 8 lanes per Jacobi pair, at least one thread per register tile of the products,
+  // and no more, since all but the pivots' warp wait through the factorisations: with 256 threads at
+  // CHI = 16 three realizations fit on an SM and issued 1.1 instructions a cycle between them.
+  static constexpr int NT = 8 * CHI;
+  static constexpr int NWARP = NT / 32;
+  // Realizations per SM that the FP32 registers are cut to (shared memory allows three at CHI = 32),
+  // and the runs of the factorisations.  CHI = 16 has two builds: five per SM with short runs for a
+  // few realizations, seven with long ones (72 registers, a fifth less code: with more blocks in
+  // different phases the instruction cache is what they wait for) for a crowd.  16 x 16 lattices, ms
+  // by realizations: 100 9.5 / 10.8, 760 13.3 / 14.3, 1064 24.4 / 17.7, 1520 27.5 / 30.8.
+  static constexpr int PER_SM = CHI > 32 ? 1 : (CHI == 32 ? 3 : (CHI == 16 ? (kCrowd ? 7 : 5) : (CHI == 8 ? 8 : 16)));
+  static constexpr int RUN = kCrowd ? 8 : 4;
+  // The sum of Y's squares is associated as VT threads' partial sums, whatever NT: it is the scale
+  // that Jacobi's threshold hangs on.
+  static constexpr int VT = CHI > 32 ? 512 : (CHI > 4 ? 256 : 128);
   static constexpr int TILE = 2 * CHI * CHI;        // [y][alpha][beta]
 };
 
@@ -165,9 +175,9 @@ template <typename T, int CHI> struct JStride {
 
 template <typename T, int CHI>
 __host__ __device__ constexpr size_t env_smem_elems() {
-  // CHI = 64: only Y and V (D*DP each) and the reflector slots (16 of 2D) stay in shared memory;
+  // CHI = 64: only Y and V (D*DP each) stay in shared memory;
   // M lives in per-realization global scratch and R, the tile are read from global memory
-  if (CHI > 32) return (size_t)2 * (2 * CHI) * JStride<T, CHI>::DP + (size_t)32 * (2 * CHI);
+  if (CHI > 32) return (size_t)2 * (2 * CHI) * JStride<T, CHI>::DP;
   // backward: M, R (D*D each), Y, V (D*DP each) + tile (2*CHI*CHI); P (D*CHI) lives in the Y
   //           region and Q (2*CHI*CHI) in the V region between their uses
   // forward : X (2D*D, aliases M and Y) + R (D*D) + tile; the Householder vectors use V
@@ -186,22 +196,23 @@ __host__ __device__ constexpr size_t env_smem_elems() {
 // l = g mod G, so the levels down to G are register adds and only log2(G) shuffles remain.
 //
 // What bounds it: the chain dot product -> shuffles -> update -> norm -> square root -> publish of
-// consecutive pivots (about 700 cycles each at 64 x 64, 520 in one warp), not the arithmetic.  With the
+// consecutive pivots (about 690 cycles each at 64 x 64, 400 in one warp), not the arithmetic.  With the
 // columns in shared memory a reflector cost 1440 cycles: every step read and wrote the whole matrix
 // there and reduced each dot product over 32 lanes, 870 cycles of the shared-memory pipe alone.
 // 16 rows a lane and log2(MR/16) shuffle levels balance the serial adds of a lane against the
 // shuffles (30 cycles a level).  Environment build at chi = 32, FP32 (one GB300): 203 -> 150 us a site
 // step with one realization per SM (L = 64), 331 -> 214 us with three (L = 48).
-template <typename T, int MR, int NC> struct QrCfg {
+template <typename T, int MR, int NC, int KR> struct QrCfg {
   static constexpr int G = MR >= 32 ? MR / 16 : 2;          // lanes of a column: 16 rows each from MR = 32 on
   static constexpr int RPT = MR / G;
   static constexpr int NVL = 32 / G < RPT ? 32 / G : RPT;   // partial sums a lane holds
-  static constexpr int NRUN = RPT / 4;                      // runs of four rows a lane holds
+  // The factorisation has one body for each run of KR rows of a lane (the pivots whose rows are in
+  // it; the rows of earlier runs are left out): short runs save products of zeros and cost code.
+  static constexpr int RUN = RPT < KR ? RPT : KR;
   static constexpr int CPT = NC * G > 512 ? (NC * G) / 512 : (NC * G > 256 ? 2 : 1);
   static constexpr int NTQ = NC * G / CPT < 32 ? 32 : NC * G / CPT;   // threads taking part
   static constexpr int GPW = 32 / G;                        // groups of a warp
   static constexpr int CW = GPW * CPT;                      // columns of a warp
-  static constexpr int RING = NTQ == 32 ? 2 : 16;           // reflector slots in turn
 };
 // Place of row i in a column stored for QrCfg: each lane's rows in 16-byte runs of four, the runs of
 // the G lanes side by side, so that a group reads its column in conflict-free vector loads.
@@ -245,7 +256,7 @@ __device__ __forceinline__ T qr_dot(const T (&v)[Q::RPT], const T (&x)[Q::RPT]) 
 #pragma unroll
   for (int a = 0; a < Q::NVL; ++a) p[a] = T(0);
 #pragma unroll
-  for (int u = 4 * C0; u < Q::RPT; u += 2) fma_pair(v + u, x + u, p + u % Q::NVL);
+  for (int u = Q::RUN * C0; u < Q::RPT; u += 2) fma_pair(v + u, x + u, p + u % Q::NVL);
 #pragma unroll
   for (int lv = Q::NVL / 2; lv > 1; lv >>= 1)
 #pragma unroll
@@ -259,26 +270,39 @@ template <typename Q, int C0, typename T>
 __device__ __forceinline__ void qr_update(T md, const T (&v)[Q::RPT], T (&x)[Q::RPT]) {
   const T m2[2] = {md, md};
 #pragma unroll
-  for (int u = 4 * C0; u < Q::RPT; u += 2) fma_pair(m2, v + u, x + u);
+  for (int u = Q::RUN * C0; u < Q::RPT; u += 2) fma_pair(m2, v + u, x + u);
 }
 template <typename Q, int C0, typename T>
 __device__ __forceinline__ void qr_load_v(const T* vs, int g, T (&v)[Q::RPT]) {
 #pragma unroll
-  for (int ch = C0; ch < Q::NRUN; ++ch) ld4(vs + ch * 4 * Q::G + g * 4, v + 4 * ch);
+  for (int u = Q::RUN * C0; u < Q::RPT; u += 4) ld4(vs + u * Q::G + g * 4, v + u);
 }
-__device__ __forceinline__ void named_arrive(int id, int nthreads) {
-  asm volatile("bar.arrive %0, %1;\n" ::"r"(id), "r"(nthreads) : "memory");
+// Named barrier 3 + k (k < 4), waited for or only arrived at.  The number is spelled out in the
+// instruction: with one in a register the compiler reserves all 16 barriers for the block, and an SM's
+// 64 then hold four blocks.
+__device__ __forceinline__ void turn_sync(int k, int n) {
+  if (k & 2) {
+    if (k & 1) asm volatile("bar.sync 6, %0;\n" ::"r"(n) : "memory");
+    else asm volatile("bar.sync 5, %0;\n" ::"r"(n) : "memory");
+  } else {
+    if (k & 1) asm volatile("bar.sync 4, %0;\n" ::"r"(n) : "memory");
+    else asm volatile("bar.sync 3, %0;\n" ::"r"(n) : "memory");
+  }
+}
+__device__ __forceinline__ void turn_arrive(int k, int n) {        // k = 0, 1, 2
+  if (k & 2) asm volatile("bar.arrive 5, %0;\n" ::"r"(n) : "memory");
+  else if (k & 1) asm volatile("bar.arrive 4, %0;\n" ::"r"(n) : "memory");
+  else asm volatile("bar.arrive 3, %0;\n" ::"r"(n) : "memory");
 }
 
 // State of one factorisation: where the reflectors go and how they are handed on.
-// The warp that owns the pivot columns runs ahead: it publishes reflector after reflector with
-// bar.arrive and only the others wait.  The published reflectors use eight barriers in turn, and
-// with every eighth the pivot's warp waits too, so that no barrier is used again before all have
-// passed it; the reflector slots (16 in turn unless all are kept) follow from the same count: a slot is
-// written again only after a barrier that all have passed since they read it.
+// The warp that owns the pivot columns runs ahead: it publishes reflector after reflector, each in a
+// slot of its own, and only arrives at that reflector's barrier while the others wait.  The published
+// reflectors use four barriers in turn, and with every fourth the pivot's warp waits too, so that no
+// barrier is used again before all have passed it.  (Flags in shared memory that the others poll
+// took their issue slots: 459 instead of 388 ms at three CTAs per SM.)
 template <typename T> struct QrOut {
-  T* vring;          // slots of MR elements
-  bool keep_all;     // slot j holds reflector j, else published reflector k is in slot k mod RING
+  T* v;              // slot j (MR elements): reflector j
   T* vsave;          // the reflectors once more, at j * MR (nullable)
   T* cden;           // [j]: reflector j's coefficient 2/|v|^2 (0: no reflector), with kLate its reciprocal
   T* diag;           // [j]: R_jj
@@ -287,25 +311,35 @@ template <typename T> struct QrOut {
 // where a division occupies the FP64 pipe, only the pivot's warp does.
 template <typename T> constexpr bool kLate = sizeof(T) == 4;
 
+// 1 / x, correctly rounded for normal x and 1 / x: the hardware's approximation and one Newton step with
+// a fused residual (Markstein 1990), checked against the division for every float in [1e-37, 1e37].
+// The division's branch for its special cases keeps it from overlapping with the dot products.
+__device__ __forceinline__ float inverse(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return fmaf(r, fmaf(-x, r, 1.0f), r);
+}
+__device__ __forceinline__ double inverse(double x) { return 1.0 / x; }
+
 // Reflector of column j, by the warp that owns it; j lies in the rows of run C0.
-template <typename T, int MR, int NC, int C0>
-__device__ __forceinline__ void qr_pivot(T (&x)[QrCfg<T, MR, NC>::CPT][QrCfg<T, MR, NC>::RPT], int j, T* vs,
+template <typename T, int MR, int NC, int KR, int C0>
+__device__ __forceinline__ void qr_pivot(T (&x)[QrCfg<T, MR, NC, KR>::CPT][QrCfg<T, MR, NC, KR>::RPT], int j, T* vs,
                                          const QrOut<T>& o, int g, int gi, int warp) {
-  using Q = QrCfg<T, MR, NC>;
+  using Q = QrCfg<T, MR, NC, KR>;
   constexpr int G = Q::G;
   const T tiny = (sizeof(T) == 4) ? T(1e-36) : T(1e-300);
-  const int jl = j - warp * Q::CW, jq = jl / Q::GPW, jr = j - 4 * G * C0;   // row of the pivot within the run
+  const int jl = j - warp * Q::CW, jq = jl / Q::GPW, jr = j - Q::RUN * G * C0;   // row of the pivot within the run
 #pragma unroll
   for (int q = 0; q < Q::CPT; ++q) {
     if (Q::CPT > 1 && q != jq) continue;     // warp-uniform
     T xr[Q::RPT], x0 = T(0);
 #pragma unroll
-    for (int u = 4 * C0; u < Q::RPT; ++u) xr[u] = x[q][u];
+    for (int u = Q::RUN * C0; u < Q::RPT; ++u) xr[u] = x[q][u];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
+    for (int u = 0; u < Q::RUN; ++u) {
       const int i = g + G * u;               // rows above the pivot belong to R
-      if (i < jr) xr[4 * C0 + u] = T(0);
-      if (i == jr) x0 = xr[4 * C0 + u];
+      if (i < jr) xr[Q::RUN * C0 + u] = T(0);
+      if (i == jr) x0 = xr[Q::RUN * C0 + u];
     }
     const T ss = qr_dot<Q, C0, T>(xr, xr);
     const bool null = ss <= tiny;
@@ -314,12 +348,12 @@ __device__ __forceinline__ void qr_pivot(T (&x)[QrCfg<T, MR, NC>::CPT][QrCfg<T, 
       const T alpha = x0 >= T(0) ? -nrm : nrm;
       const T v0 = x0 - alpha;
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (g + G * u == jr) { xr[4 * C0 + u] = v0; if (!null) x[q][4 * C0 + u] = alpha; }
+      for (int u = 0; u < Q::RUN; ++u)
+        if (g + G * u == jr) { xr[Q::RUN * C0 + u] = v0; if (!null) x[q][Q::RUN * C0 + u] = alpha; }
 #pragma unroll
-      for (int ch = C0; ch < Q::NRUN; ++ch) {
-        st4(vs + ch * 4 * G + g * 4, xr + 4 * ch);
-        if (o.vsave) st4(o.vsave + (size_t)j * MR + ch * 4 * G + g * 4, xr + 4 * ch);
+      for (int u = Q::RUN * C0; u < Q::RPT; u += 4) {
+        st4(vs + u * G + g * 4, xr + u);
+        if (o.vsave) st4(o.vsave + (size_t)j * MR + u * G + g * 4, xr + u);
       }
       if (g == jr % G) {
         const T den = nrm * (nrm + (x0 >= T(0) ? x0 : -x0));
@@ -331,26 +365,30 @@ __device__ __forceinline__ void qr_pivot(T (&x)[QrCfg<T, MR, NC>::CPT][QrCfg<T, 
 }
 
 // The pivots whose rows lie in run C0, then those of the later runs.
-template <typename T, int MR, int NC, int C0, typename Skip>
-__device__ __forceinline__ void qr_runs(T (&x)[QrCfg<T, MR, NC>::CPT][QrCfg<T, MR, NC>::RPT], int nc, int& pub,
+template <typename T, int MR, int NC, int KR, int C0, typename Skip>
+__device__ __forceinline__ void qr_runs(T (&x)[QrCfg<T, MR, NC, KR>::CPT][QrCfg<T, MR, NC, KR>::RPT], int nc, int& pub,
                                         const QrOut<T>& o, int g, int gi, int warp, Skip skip) {
-  using Q = QrCfg<T, MR, NC>;
-  constexpr int J0 = 4 * Q::G * C0, J1 = J0 + 4 * Q::G < NC ? J0 + 4 * Q::G : NC;
-  auto slot = [&](int j) { return o.vring + (size_t)(o.keep_all ? j : pub % Q::RING) * MR; };
+  using Q = QrCfg<T, MR, NC, KR>;
+  constexpr int J0 = Q::RUN * Q::G * C0, J1 = J0 + Q::RUN * Q::G < NC ? J0 + Q::RUN * Q::G : NC;
   const int first = warp * Q::CW, last = first + Q::CW - 1;
   const int je = nc < J1 ? nc : J1;
-  if (J0 < je && J0 >= first && J0 <= last && !skip(J0)) qr_pivot<T, MR, NC, C0>(x, J0, slot(J0), o, g, gi, warp);
   for (int j = J0; j < je; ++j) {
-    const bool live = !skip(j);
-    if (live) {
-      if constexpr (Q::NTQ == 32) __syncwarp();
-      else if (j >= first && j <= last && (pub & 7) != 7) { __syncwarp(); named_arrive(2 + (pub & 7), Q::NTQ); }
-      else named_barrier(2 + (pub & 7), Q::NTQ);
+    if (!skip(j)) {
+      if (j >= first && j <= last) qr_pivot<T, MR, NC, KR, C0>(x, j, o.v + (size_t)j * MR, o, g, gi, warp);
+      if constexpr (Q::NTQ == 32) {
+        __syncwarp();
+      } else if (j >= first && j <= last && (pub & 3) != 3) {
+        __syncwarp();
+        turn_arrive(pub & 3, Q::NTQ);
+      } else {
+        turn_sync(pub & 3, Q::NTQ);
+      }
+      ++pub;
       if (last > j) {
         T v[Q::RPT];
-        qr_load_v<Q, C0, T>(slot(j), g, v);
+        qr_load_v<Q, C0, T>(o.v + (size_t)j * MR, g, v);
         const T den = o.cden[j];
-        const T coef = !kLate<T> || den == T(0) ? den : T(1) / den;
+        const T coef = !kLate<T> || den == T(0) ? den : inverse(den);
 #pragma unroll
         for (int q = 0; q < Q::CPT; ++q) {
           T d = qr_dot<Q, C0, T>(v, x[q]) * coef;
@@ -358,30 +396,27 @@ __device__ __forceinline__ void qr_runs(T (&x)[QrCfg<T, MR, NC>::CPT][QrCfg<T, M
           qr_update<Q, C0>(-d, v, x[q]);
         }
       }
-      ++pub;
     }
-    const int nx = j + 1;
-    if (nx < je && nx >= first && nx <= last && !skip(nx)) qr_pivot<T, MR, NC, C0>(x, nx, slot(nx), o, g, gi, warp);
   }
-  if constexpr (J1 < NC) qr_runs<T, MR, NC, C0 + 1>(x, nc, pub, o, g, gi, warp, skip);
+  if constexpr (J1 < NC) qr_runs<T, MR, NC, KR, C0 + 1>(x, nc, pub, o, g, gi, warp, skip);
 }
 
 // Factor the columns j < nc for which skip(j) is false (skip(j): the column is known to be zero, so
 // its reflector is the identity; it must be the same for every thread).  On return x holds R on and
 // above the diagonal (below it, what is left of the reflectors).
-template <typename T, int MR, int NC, typename Skip>
-__device__ __forceinline__ void qr_factor(T (&x)[QrCfg<T, MR, NC>::CPT][QrCfg<T, MR, NC>::RPT], int nc,
+template <typename T, int MR, int NC, int KR, typename Skip>
+__device__ __forceinline__ void qr_factor(T (&x)[QrCfg<T, MR, NC, KR>::CPT][QrCfg<T, MR, NC, KR>::RPT], int nc,
                                           const QrOut<T>& o, int lane, int warp, Skip skip) {
-  using Q = QrCfg<T, MR, NC>;
+  using Q = QrCfg<T, MR, NC, KR>;
   int pub = 0;                              // reflectors published
-  qr_runs<T, MR, NC, 0>(x, nc, pub, o, lane % Q::G, lane / Q::G, warp, skip);
+  qr_runs<T, MR, NC, KR, 0>(x, nc, pub, o, lane % Q::G, lane / Q::G, warp, skip);
 }
 
 // x <- H_0 H_1 ... H_{n-1} x for one column per group, the reflectors as qr_factor kept them.
-template <typename T, int MR, int NC, int C0 = (NC - 1) / (4 * QrCfg<T, MR, NC>::G)>
-__device__ __forceinline__ void qr_apply_q(T (&x)[QrCfg<T, MR, NC>::RPT], int n, const T* vs, const T* coefs, int g) {
-  using Q = QrCfg<T, MR, NC>;
-  constexpr int J0 = 4 * Q::G * C0, J1 = J0 + 4 * Q::G < NC ? J0 + 4 * Q::G : NC;
+template <typename T, int MR, int NC, int KR, int C0 = (NC - 1) / (QrCfg<T, MR, NC, KR>::RUN * QrCfg<T, MR, NC, KR>::G)>
+__device__ __forceinline__ void qr_apply_q(T (&x)[QrCfg<T, MR, NC, KR>::RPT], int n, const T* vs, const T* coefs, int g) {
+  using Q = QrCfg<T, MR, NC, KR>;
+  constexpr int J0 = Q::RUN * Q::G * C0, J1 = J0 + Q::RUN * Q::G < NC ? J0 + Q::RUN * Q::G : NC;
   for (int j = (n < J1 ? n : J1) - 1; j >= J0; --j) {
     const T coef = coefs[j];
     if (coef == T(0)) continue;
@@ -390,13 +425,13 @@ __device__ __forceinline__ void qr_apply_q(T (&x)[QrCfg<T, MR, NC>::RPT], int n,
     const T d = qr_dot<Q, C0, T>(v, x) * coef;
     qr_update<Q, C0>(-d, v, x);
   }
-  if constexpr (C0 > 0) qr_apply_q<T, MR, NC, C0 - 1>(x, n, vs, coefs, g);
+  if constexpr (C0 > 0) qr_apply_q<T, MR, NC, KR, C0 - 1>(x, n, vs, coefs, g);
 }
 
-template <typename T, typename TE, int CHI>
-__global__ void __launch_bounds__(EnvCfg<CHI>::NT, (sizeof(T) == 8 || CHI > 32) ? 1 : 3)
+template <typename T, typename TE, int CHI, bool kCrowd>
+__global__ void __launch_bounds__(EnvCfg<CHI>::NT, sizeof(T) == 8 ? 1 : EnvCfg<CHI, kCrowd>::PER_SM)
 env_build_kernel(EnvBuildArgs<T, TE> args) {
-  using C = EnvCfg<CHI>;
+  using C = EnvCfg<CHI, kCrowd>;
   constexpr int D = C::D, NWARP = C::NWARP, NT = C::NT, TILE = C::TILE;
   const int L = args.L;
   const int real = blockIdx.x;
@@ -426,13 +461,11 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
   T* Xs = sm;                 // 2D x D col-major
 
   __shared__ T Wc[8];               // W[x][a][b] at x*4 + a*2 + b
-  int8_t* jv_s = reinterpret_cast<int8_t*>(kBig ? Vc + D * DP + 32 * D : Bt + TILE);   // Jv[r][c], L entries
+  int8_t* jv_s = reinterpret_cast<int8_t*>(kBig ? Vc + D * DP : Bt + TILE);   // Jv[r][c], L entries
   int8_t* jh_s = jv_s + args.L;                                // Jh[r+1][c], L-1 entries
   const T eb = (T)exp(beta), ebm = (T)exp(-beta);             // exp(+-beta): every Boltzmann weight
-  using QF = QrCfg<T, 2 * D, D>;     // the forward sweep's QR
-  using QB = QrCfg<T, D, D>;         // the backward sweep's
-  // reflector slots (the V region is idle in the forward sweep unless X fills Y and V, as for kBig)
-  T* const vfwd = kBig ? Vc + D * DP : Vc;
+  using QF = QrCfg<T, 2 * D, D, C::RUN>;     // the forward sweep's QR
+  using QB = QrCfg<T, D, D, C::RUN>;         // the backward sweep's
   __shared__ T csave[D];            // the reflectors' coefficients (as qr_factor leaves them, then inverted)
   __shared__ T diag[D];
   __shared__ T red[32];
@@ -578,8 +611,11 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
         // columns (b, be) beyond the right bond of the previous row's tile are zero
         const int kr = kold[c + 1];
         auto zero_col = [&](int j) { return (j & (CHI - 1)) >= kr; };
-        const QrOut<T> out{vfwd, false, nullptr, csave, diag};
-        qr_factor<T, 2 * D, D>(x, D, out, lane, warp, zero_col);
+        // the reflectors take X's place, column by column of it read by now
+        if constexpr (QF::NTQ == 32) __syncwarp();
+        else named_barrier<2>(QF::NTQ);
+        const QrOut<T> out{Xs, nullptr, csave, diag};
+        qr_factor<T, 2 * D, D, C::RUN>(x, D, out, lane, warp, zero_col);
         T mx = 0;
         for (int j = lane; j < D; j += 32)
           if (!zero_col(j)) { const T v = diag[j] < 0 ? -diag[j] : diag[j]; mx = v > mx ? v : mx; }
@@ -659,7 +695,7 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
       // M[(a,al)][j] = sum_b W(x,a,b) Q[b][al][g]
       for (int e = tid; e < D * n; e += NT) {
         const int row = e % D, j = e / D;
-        const int a = row / CHI, al = row % CHI, x = j / kn, g = j % kn;
+        const int a = row / CHI, al = row % CHI, x = j >= kn, g = j - x * kn;
         Mc[e] = Wc[x * 4 + a * 2 + 0] * Qs[0 * CHI * CHI + al * CHI + g] +
                 Wc[x * 4 + a * 2 + 1] * Qs[1 * CHI * CHI + al * CHI + g];
       }
@@ -691,13 +727,15 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
       // Y = R_c M  (D x n; R_c, the R factor of the left part up to site c-1, was
       // prefetched): 4 x 4 register tiles over (rows, compact columns).  Zip-up: Y = M (the
       // previous row is canonical on the side not yet swept, so no R factor)
-      T fro = 0;
+      constexpr int VK = C::VT / NT;
+      T fro[VK] = {};
       if (zip) {
         for (int e = tid; e < DP * n; e += NT) {
           const int i = e % DP, j = e / DP;
           const T v = i < D ? Mc[(size_t)j * D + i] : T(0);
           Yc[e] = v;
-          fro += v * v;
+#pragma unroll
+          for (int q = 0; q < VK; ++q) if ((e / NT) % VK == q) fro[q] += v * v;
         }
       } else {
         constexpr int TI = D / 4;
@@ -722,7 +760,8 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
 #pragma unroll
               for (int ii = 0; ii < 4; ++ii) {
                 Yc[(size_t)(j0 + jj) * DP + qr_pos<QB::G>(i0 + ii)] = acc[ii][jj];
-                fro += acc[ii][jj] * acc[ii][jj];
+#pragma unroll
+                for (int q = 0; q < VK; ++q) if ((u / NT) % VK == q) fro[q] += acc[ii][jj] * acc[ii][jj];
               }
             }
           }
@@ -731,17 +770,20 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
       // the Jacobi runs on npad = n rounded up to 8 columns (blocks of 4, an even number of
       // blocks); columns n..npad-1 of Y are zero and never rotate
       const int npad = (n + 7) & ~7;
-      fro = warp_sum(fro);
-      if (lane == 0) red[warp] = fro;
+#pragma unroll
+      for (int q = 0; q < VK; ++q) {
+        const T f = warp_sum(fro[q]);
+        if (lane == 0) red[q * NWARP + warp] = f;
+      }
       if (tid == 0) { rot[0] = 0; rot[1] = 0; rot[2] = 0; }
       __syncthreads();
       if (warp == 0) {
-        T f = lane < NWARP ? red[lane] : T(0);
+        T f = lane < C::VT / 32 ? red[lane] : T(0);
         f = warp_sum(f);
-        if (lane == 0) red[NWARP] = f;
+        if (lane == 0) red[C::VT / 32] = f;
       }
       __syncthreads();
-      const T tinyY = red[NWARP] * num<T>::eps * num<T>::eps;
+      const T tinyY = red[C::VT / 32] * num<T>::eps * num<T>::eps;
       if (zip) {
         // the zip-up's Y = M is graded by columns (P = U S), where the one-sided Jacobi is
         // accurate without preconditioning
@@ -770,37 +812,33 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
           }
         };
         if (warp < QB::NTQ / 32) {
-          load(Yc);
-          if constexpr (QB::NTQ == 32) __syncwarp();
-          else named_barrier(10, QB::NTQ);
-          const QrOut<T> out1{kBig ? vfwd : Yc, false, nullptr, csave, diag};
-          qr_factor<T, D, D>(x, n, out1, lane, warp, none);
+          // one body for both; pass 0: Y, its reflectors in Y's place, R1^T to V (stored for the next
+          // pass); pass 1: R1^T, the reflectors in R_c's place (CHI = 64: in V's and saved to R_c),
+          // R2^T to Y, zero outside n x n
+#pragma unroll 1
+          for (int pass = 0; pass < 2; ++pass) {
+            load(pass ? Vc : Yc);
+            if (pass == 0 || kBig) {                         // the reflectors take the place of what is read
+              if constexpr (QB::NTQ == 32) __syncwarp();
+              else named_barrier<2>(QB::NTQ);
+            }
+            const QrOut<T> out{pass ? (kBig ? Vc : Rc) : Yc, pass && kBig ? Rc : nullptr, csave, diag};
+            qr_factor<T, D, D, C::RUN>(x, n, out, lane, warp, none);
+            T* const to = pass ? Yc : Vc;
 #pragma unroll
-          for (int q = 0; q < QB::CPT; ++q) {                // R1^T, stored for the next factorisation
-            const int col = warp * QB::CW + q * QB::GPW + gi;
-            if (col < D) {
+            for (int q = 0; q < QB::CPT; ++q) {
+              const int col = warp * QB::CW + q * QB::GPW + gi;
+              const int at = pass ? col : qr_pos<QB::G>(col);
+              if (col < D) {
 #pragma unroll
-              for (int u = 0; u < QB::RPT; ++u) {
-                const int i = g + QB::G * u;
-                Vc[(size_t)i * DP + qr_pos<QB::G>(col)] = (i <= col && col < n) ? x[q][u] : T(0);
+                for (int u = 0; u < QB::RPT; ++u) {
+                  const int i = g + QB::G * u;
+                  to[(size_t)i * DP + at] = (i <= col && col < n) ? x[q][u] : T(0);
+                }
               }
             }
-          }
-          if constexpr (QB::NTQ == 32) __syncwarp();
-          else named_barrier(10, QB::NTQ);
-          load(Vc);
-          const QrOut<T> out2{kBig ? vfwd : Rc, !kBig, kBig ? Rc : nullptr, csave, diag};
-          qr_factor<T, D, D>(x, n, out2, lane, warp, none);
-#pragma unroll
-          for (int q = 0; q < QB::CPT; ++q) {                // R2^T in Y, zero outside n x n
-            const int col = warp * QB::CW + q * QB::GPW + gi;
-            if (col < D) {
-#pragma unroll
-              for (int u = 0; u < QB::RPT; ++u) {
-                const int i = g + QB::G * u;
-                Yc[(size_t)i * DP + col] = (i <= col && col < n) ? x[q][u] : T(0);
-              }
-            }
+            if constexpr (QB::NTQ == 32) __syncwarp();
+            else named_barrier<2>(QB::NTQ);
           }
           if constexpr (DP > D)
             for (int e = tid; e < (DP - D) * D; e += QB::NTQ) Yc[(size_t)(e / (DP - D)) * DP + D + e % (DP - D)] = T(0);
@@ -872,7 +910,7 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
           sum8(a, 2);
           if (li == 0) n2[p0 + grp] = a[0] > a[1] ? a[0] : a[1];
         }
-        named_barrier(1, NJ);
+        named_barrier<1>(NJ);
         bool live = false;
         if (lane < NB) {
 #pragma unroll
@@ -985,7 +1023,7 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
                 }
               }
             }
-            named_barrier(1, NJ);
+            named_barrier<1>(NJ);
           }
           if (rot[sweep % 3] == 0) break;
         }
@@ -1031,7 +1069,7 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
         }
         __syncthreads();
         if (warp * QB::GPW < k) {
-          qr_apply_q<T, D, D>(xz, n, Rc, csave, g);
+          qr_apply_q<T, D, D, C::RUN>(xz, n, Rc, csave, g);
 #pragma unroll
           for (int u = 0; u < QB::RPT; ++u) {
             const int i = g + QB::G * u;
@@ -1205,15 +1243,30 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
   }
 }
 
-template <typename T, typename TE, int CHI>
-cudaError_t launch_env_build_t(const EnvBuildArgs<T, TE>& a, cudaStream_t st) {
-  using C = EnvCfg<CHI>;
+template <typename T, typename TE, int CHI, bool kCrowd>
+static cudaError_t env_build_setup(int L, size_t* smem) {
   // + the two rows' couplings (int8) staged behind the tile
-  const size_t smem = env_smem_elems<T, CHI>() * sizeof(T) + (size_t)2 * a.L + 16;
-  cudaError_t e = cudaFuncSetAttribute(env_build_kernel<T, TE, CHI>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  *smem = env_smem_elems<T, CHI>() * sizeof(T) + (size_t)2 * L + 16;
+  return cudaFuncSetAttribute(env_build_kernel<T, TE, CHI, kCrowd>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)*smem);
+}
+
+template <typename T, typename TE, int CHI, bool kCrowd = false>
+static cudaError_t launch_env_build_t(const EnvBuildArgs<T, TE>& a, cudaStream_t st) {
+  if constexpr (CHI == 16 && sizeof(T) == 4 && !kCrowd) {
+    // The crowd's build takes 4/3 of the time a full wave and holds 7/5 of the realizations: it is
+    // the shorter one where it saves waves.
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const int few = sms * EnvCfg<CHI, false>::PER_SM, many = sms * EnvCfg<CHI, true>::PER_SM;
+    if (4 * ((a.n_real + many - 1) / many) < 3 * ((a.n_real + few - 1) / few)) return launch_env_build_t<T, TE, CHI, true>(a, st);
+  }
+  size_t smem = 0;
+  const cudaError_t e = env_build_setup<T, TE, CHI, kCrowd>(a.L, &smem);
   if (e != cudaSuccess) return e;
-  env_build_kernel<T, TE, CHI><<<a.n_real, C::NT, smem, st>>>(a);
+  env_build_kernel<T, TE, CHI, kCrowd><<<a.n_real, EnvCfg<CHI>::NT, smem, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -1237,12 +1290,10 @@ template cudaError_t launch_env_build<float, __nv_bfloat16>(const EnvBuildArgs<f
 
 template <typename T, typename TE, int CHI>
 static cudaError_t occupancy_t(int L, int* per_sm) {
-  using C = EnvCfg<CHI>;
-  const size_t smem = env_smem_elems<T, CHI>() * sizeof(T) + (size_t)2 * L + 16;
-  cudaError_t e = cudaFuncSetAttribute(env_build_kernel<T, TE, CHI>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  size_t smem = 0;
+  const cudaError_t e = env_build_setup<T, TE, CHI, false>(L, &smem);
   if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, env_build_kernel<T, TE, CHI>, C::NT, smem);
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(per_sm, env_build_kernel<T, TE, CHI, false>, EnvCfg<CHI>::NT, smem);
 }
 
 cudaError_t env_build_occupancy(int L, int CHI, int precision, int* per_sm) {

@@ -42,3 +42,22 @@ def test_log_z_at_tile_edges(tn, precision, tol, compression, L, chi):
         dims = ctx.copy_env(k, 0)[1]
         assert list(dims) == env.bond_dims(0)
     ctx.close()
+
+
+@pytest.mark.parametrize("chi,compression", [(13, "canonical"), (16, "canonical"), (16, "zipup")])
+def test_same_bits_alone_and_in_a_crowd(tn, chi, compression):
+    """chi = 16 has a second build for calls whose realizations fill the GPU; a realization's
+    environments do not depend on which one it went through."""
+    L, p = 9, 0.109
+    per_sm, sms = tn.env_build_occupancy(L, chi, "fp32")
+    many = list(range(100, 100 + (per_sm + 1) * sms))       # one wave more than the other build holds
+    out = []
+    for seeds in (many, many[:3]):
+        ctx = tn.TNMC(L, tn.couplings_pmj(L, seeds, p), lattice.nishimori_beta(p), seeds, chi, precision="fp32",
+                      compression=compression)
+        lz = ctx.build_env()
+        out.append((lz[:3], [ctx.copy_env(k, r)[0] for k in range(3) for r in (0, L // 2)]))
+        ctx.close()
+    assert np.array_equal(out[0][0], out[1][0])
+    for a, b in zip(out[0][1], out[1][1]):
+        assert np.array_equal(a, b)
