@@ -646,7 +646,23 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
       Ps[e] = (g == 0 && (row % CHI) == 0) ? T(1) : T(0);
     }
     int kn = 1;             // k_{c+1}
+    // The removed scales' logarithms, added in site order.  One lane of warp 0 keeps each scale and the
+    // logarithms are taken 32 at a time: one thread's FP64 logarithm held the site up for 2400 cycles.
     double logs = 0.0;
+    T scale = T(1);
+    int n_scales = 0;
+    auto flush_scales = [&]() {
+      const double l = lane < n_scales && scale > T(0) ? log((double)scale) : 0.0;
+      for (int i = 0; i < n_scales; ++i) {
+        const double li = __shfl_sync(0xffffffffu, l, i);
+        if (__shfl_sync(0xffffffffu, scale, i) > T(0)) logs += li;
+      }
+      n_scales = 0;
+    };
+    auto keep_scale = [&](T v) {               // by the whole of warp 0
+      if (lane == n_scales) scale = v;
+      if (++n_scales == 32) flush_scales();
+    };
     if (tid == 0) knew[L] = 1;
     __syncthreads();
     for (int c = L - 1; c >= 0; --c) {
@@ -720,7 +736,8 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
           ctile0[e] = v;
           etile0[e] = env_store<TE, T>(v);
         }
-        if (tid == 0) { logs += log((double)nrm); knew[0] = 1; knew[L] = 1; }
+        if (warp == 0) { flush_scales(); logs += log((double)nrm); }
+        if (tid == 0) { knew[0] = 1; knew[L] = 1; }
         __syncthreads();
         break;
       }
@@ -777,13 +794,7 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
       }
       if (tid == 0) { rot[0] = 0; rot[1] = 0; rot[2] = 0; }
       __syncthreads();
-      if (warp == 0) {
-        T f = lane < C::VT / 32 ? red[lane] : T(0);
-        f = warp_sum(f);
-        if (lane == 0) red[C::VT / 32] = f;
-      }
-      __syncthreads();
-      const T tinyY = red[C::VT / 32] * num<T>::eps * num<T>::eps;
+      const T tinyY = warp_sum(lane < C::VT / 32 ? red[lane] : T(0)) * num<T>::eps * num<T>::eps;
       if (zip) {
         // the zip-up's Y = M is graded by columns (P = U S), where the one-sided Jacobi is
         // accurate without preconditioning
@@ -1077,11 +1088,11 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
           }
         }
         __syncthreads();
-        if (tid < k) sel[tid] = tid;
-        __syncthreads();
         // R_{c-1} streams in while the tile and P are formed (the reflectors are consumed)
         if (!kBig && c > 1) prefetch_async(Rc, Rstore + (size_t)(c - 1) * D * D, D * D * (int)sizeof(T), tid, NT);
       }
+      // column of the g-th singular vector (already gathered unless zip-up)
+      auto vcol = [&](int g) { return zip ? sel[g] : g; };
       // B_r[c][y][al][be] = V[(y,be)][sel[al]]
       T* ctile = cur + (size_t)osite(c) * TILE;
       TE* etile = erow + (size_t)osite(c) * TILE;
@@ -1089,55 +1100,52 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
         const int y = e / (CHI * CHI), i = (e / CHI) % CHI, j = e % CHI;
         const int al = mir ? j : i, be = mir ? i : j;       // frame bonds of lattice entry (i, j)
         T v = T(0);
-        if (al < k && be < kn) v = Vc[(size_t)sel[al] * DP + y * kn + be];
+        if (al < k && be < kn) v = Vc[(size_t)vcol(al) * DP + y * kn + be];
         ctile[e] = v;
         etile[e] = env_store<TE, T>(v);
       }
-      // P[(a,al)][g] = sum_j M[(a,al)][j] V[j][sel[g]]: 4 x 4 register tiles
-      T pmax = 0;
+      // P[(a,al)][g] = sum_j M[(a,al)][j] V[j][sel[g]]: 4 x 4 register tiles, at most one a thread,
+      // kept until the largest entry is known
       {
         constexpr int TI = D / 4, TG = CHI / 4;
-        for (int u = tid; u < TI * TG; u += NT) {
-          const int i0 = (u % TI) * 4, g0 = (u / TI) * 4;
-          T acc[4][4] = {};
-          if (g0 < k) {
-            const T* vc[4];
+        static_assert(TI * TG <= NT, "one tile of P per thread");
+        const int i0 = (tid % TI) * 4, g0 = (tid / TI) * 4;
+        const bool mine = tid < TI * TG;
+        T acc[4][4] = {}, pmax = 0;
+        if (mine && g0 < k) {
+          const T* vc[4];
 #pragma unroll
-            for (int jj = 0; jj < 4; ++jj) vc[jj] = Vc + (size_t)sel[(g0 + jj < k) ? g0 + jj : g0] * DP;
+          for (int jj = 0; jj < 4; ++jj) vc[jj] = Vc + (size_t)vcol((g0 + jj < k) ? g0 + jj : g0) * DP;
 #pragma unroll 4
-            for (int j = 0; j < n; ++j) {
-              T mv[4], vv[4];
-              ld4(Mc + (size_t)j * D + i0, mv);
+          for (int j = 0; j < n; ++j) {
+            T mv[4], vv[4];
+            ld4(Mc + (size_t)j * D + i0, mv);
 #pragma unroll
-              for (int jj = 0; jj < 4; ++jj) vv[jj] = (g0 + jj < k) ? vc[jj][j] : T(0);
+            for (int jj = 0; jj < 4; ++jj) vv[jj] = (g0 + jj < k) ? vc[jj][j] : T(0);
 #pragma unroll
-              for (int ii = 0; ii < 4; ++ii)
+            for (int ii = 0; ii < 4; ++ii)
 #pragma unroll
-                for (int jj = 0; jj < 4; ++jj) acc[ii][jj] += mv[ii] * vv[jj];
-            }
+              for (int jj = 0; jj < 4; ++jj) acc[ii][jj] += mv[ii] * vv[jj];
           }
+#pragma unroll
+          for (int ii = 0; ii < 4; ++ii)
+#pragma unroll
+            for (int jj = 0; jj < 4; ++jj) { const T aa = acc[ii][jj] < T(0) ? -acc[ii][jj] : acc[ii][jj]; pmax = aa > pmax ? aa : pmax; }
+        }
+        pmax = warp_max(pmax);
+        if (lane == 0) red[warp] = pmax;
+        __syncthreads();
+        const T pm = warp_max(lane < NWARP ? red[lane] : T(0));
+        const T pinv = pm > T(0) ? T(1) / pm : T(1);
+        if (mine) {
 #pragma unroll
           for (int jj = 0; jj < 4; ++jj) {
-            const T col4[4] = {acc[0][jj], acc[1][jj], acc[2][jj], acc[3][jj]};
+            const T col4[4] = {acc[0][jj] * pinv, acc[1][jj] * pinv, acc[2][jj] * pinv, acc[3][jj] * pinv};
             st4(Ps + (size_t)(g0 + jj) * D + i0, col4);
-#pragma unroll
-            for (int ii = 0; ii < 4; ++ii) { const T aa = acc[ii][jj] < T(0) ? -acc[ii][jj] : acc[ii][jj]; pmax = aa > pmax ? aa : pmax; }
           }
         }
+        if (warp == 0) keep_scale(pm);
       }
-      pmax = warp_max(pmax);
-      if (lane == 0) red[warp] = pmax;
-      __syncthreads();
-      if (warp == 0) {
-        T f = lane < NWARP ? red[lane] : T(0);
-        f = warp_max(f);
-        if (lane == 0) red[NWARP] = f;
-      }
-      __syncthreads();
-      const T pm = red[NWARP];
-      const T pinv = pm > T(0) ? T(1) / pm : T(1);
-      for (int e = tid; e < D * CHI; e += NT) Ps[e] *= pinv;
-      if (tid == 0 && pm > T(0)) logs += log((double)pm);
       kn = knext_s;
       __syncthreads();
     }
