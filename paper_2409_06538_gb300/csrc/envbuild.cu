@@ -456,7 +456,7 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
   // that site's Y is formed; Q is written after this site's V is dead and read before the next
   // V is initialised: so P takes the Y region and Q the V region
   T* Ps = Yc;                 // D x CHI col-major: P[(b,be)][g] at g*D + b*CHI + be
-  T* Qs = Vc;                 // 2 x CHI x CHI: Q[b][al][g]
+  T* Qs = Vc;                 // 2 x CHI x CHI: Q[b][g][al]
   // forward-phase layout (aliases M/Y/V; R stays at Rc)
   T* Xs = sm;                 // 2D x D col-major
 
@@ -678,30 +678,37 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
       // reads the previous row's tile with its bonds swapped)
       {
         constexpr int TA = CHI / 4;
-        const int sA = mir ? 1 : CHI, sB = mir ? CHI : 1;
         for (int u = tid; u < 2 * TA * TA; u += NT) {
           const int b = u / (TA * TA), a0 = ((u % (TA * TA)) % TA) * 4, g0 = ((u % (TA * TA)) / TA) * 4;
           T acc[4][4] = {};
           if (g0 < kn) {
-#pragma unroll 4
-            for (int be = 0; be < CHI; ++be) {
-              T bv[4], pv[4];
+            // four be at a time: vector loads of the rows of B (of its columns in a mirrored row) and
+            // of the columns of P
+            for (int be0 = 0; be0 < CHI; be0 += 4) {
+              T bv[4][4], pv[4][4];        // [ii][be], [jj][be]
 #pragma unroll
-              for (int ii = 0; ii < 4; ++ii) bv[ii] = Bt[b * CHI * CHI + (a0 + ii) * sA + be * sB];
+              for (int t = 0; t < 4; ++t) {
+                T v[4];
+                ld4(Bt + b * CHI * CHI + (mir ? (be0 + t) * CHI + a0 : (a0 + t) * CHI + be0), v);
 #pragma unroll
-              for (int jj = 0; jj < 4; ++jj) pv[jj] = Ps[(g0 + jj) * D + b * CHI + be];
+                for (int q = 0; q < 4; ++q) { if (mir) bv[q][t] = v[q]; else bv[t][q] = v[q]; }
+                ld4(Ps + (size_t)(g0 + t) * D + b * CHI + be0, pv[t]);
+              }
 #pragma unroll
-              for (int ii = 0; ii < 4; ++ii)
+              for (int be = 0; be < 4; ++be)
 #pragma unroll
-                for (int jj = 0; jj < 4; ++jj) acc[ii][jj] += bv[ii] * pv[jj];
+                for (int ii = 0; ii < 4; ++ii)
+#pragma unroll
+                  for (int jj = 0; jj < 4; ++jj) acc[ii][jj] += bv[ii][be] * pv[jj][be];
             }
           }
+          // Q is kept [b][g][al]: M's rows run over al
 #pragma unroll
-          for (int ii = 0; ii < 4; ++ii) {
-            T row4[4];
+          for (int jj = 0; jj < 4; ++jj) {
+            T col4[4];
 #pragma unroll
-            for (int jj = 0; jj < 4; ++jj) row4[jj] = (g0 + jj < kn) ? acc[ii][jj] : T(0);
-            st4(Qs + b * CHI * CHI + (a0 + ii) * CHI + g0, row4);
+            for (int ii = 0; ii < 4; ++ii) col4[ii] = (g0 + jj < kn) ? acc[ii][jj] : T(0);
+            st4(Qs + b * CHI * CHI + (g0 + jj) * CHI + a0, col4);
           }
         }
       }
@@ -712,8 +719,8 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
       for (int e = tid; e < D * n; e += NT) {
         const int row = e % D, j = e / D;
         const int a = row / CHI, al = row % CHI, x = j >= kn, g = j - x * kn;
-        Mc[e] = Wc[x * 4 + a * 2 + 0] * Qs[0 * CHI * CHI + al * CHI + g] +
-                Wc[x * 4 + a * 2 + 1] * Qs[1 * CHI * CHI + al * CHI + g];
+        Mc[e] = Wc[x * 4 + a * 2 + 0] * Qs[0 * CHI * CHI + g * CHI + al] +
+                Wc[x * 4 + a * 2 + 1] * Qs[1 * CHI * CHI + g * CHI + al];
       }
       __syncthreads();
       if (c == 0) {
@@ -760,16 +767,22 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
         for (int u = tid; u < TI * TJ; u += NT) {
           const int i0 = (u % TI) * 4, j0 = (u / TI) * 4;
           T acc[4][4] = {};
-#pragma unroll 4
-          for (int l = 0; l < D; ++l) {
-            T rv[4], mv[4];
-            ld4(Rc + l * D + i0, rv);
+          for (int l = 0; l < D; l += 4) {
+            T mv[4][4];
 #pragma unroll
-            for (int jj = 0; jj < 4; ++jj) mv[jj] = (j0 + jj < n) ? Mc[(size_t)(j0 + jj) * D + l] : T(0);
+            for (int jj = 0; jj < 4; ++jj) {
+              mv[jj][0] = mv[jj][1] = mv[jj][2] = mv[jj][3] = T(0);
+              if (j0 + jj < n) ld4(Mc + (size_t)(j0 + jj) * D + l, mv[jj]);
+            }
 #pragma unroll
-            for (int ii = 0; ii < 4; ++ii)
+            for (int q = 0; q < 4; ++q) {
+              T rv[4];
+              ld4(Rc + (l + q) * D + i0, rv);
 #pragma unroll
-              for (int jj = 0; jj < 4; ++jj) acc[ii][jj] += rv[ii] * mv[jj];
+              for (int ii = 0; ii < 4; ++ii)
+#pragma unroll
+                for (int jj = 0; jj < 4; ++jj) acc[ii][jj] += rv[ii] * mv[jj][q];
+            }
           }
 #pragma unroll
           for (int jj = 0; jj < 4; ++jj) {
