@@ -175,12 +175,12 @@ template <typename T, int CHI> struct JStride {
 
 template <typename T, int CHI>
 __host__ __device__ constexpr size_t env_smem_elems() {
-  // CHI = 64: only Y and V (D*DP each) stay in shared memory;
-  // M lives in per-realization global scratch and R, the tile are read from global memory
-  if (CHI > 32) return (size_t)2 * (2 * CHI) * JStride<T, CHI>::DP;
+  // CHI = 64: Y, V (D*DP each) and R (D*D) stay in shared memory (192 KB); M lives in
+  // per-realization global scratch and the tile is read from global memory
+  if (CHI > 32) return (size_t)2 * (2 * CHI) * JStride<T, CHI>::DP + (size_t)(2 * CHI) * (2 * CHI);
   // backward: M, R (D*D each), Y, V (D*DP each) + tile (2*CHI*CHI); P (D*CHI) lives in the Y
   //           region and Q (2*CHI*CHI) in the V region between their uses
-  // forward : X (2D*D, aliases M and Y) + R (D*D) + tile; the Householder vectors use V
+  // forward : X (2D*D, aliases M and Y) + R (D*D) + tile; the reflectors take X's place
   // (FP32, CHI = 32: 72 KB, so three CTAs fit on one SM)
   return (size_t)2 * (2 * CHI) * (2 * CHI) + (size_t)2 * (2 * CHI) * JStride<T, CHI>::DP +
          (size_t)2 * CHI * CHI;
@@ -303,7 +303,6 @@ __device__ __forceinline__ void turn_arrive(int k, int n) {        // k = 0, 1, 
 // took their issue slots: 459 instead of 388 ms at three CTAs per SM.)
 template <typename T> struct QrOut {
   T* v;              // slot j (MR elements): reflector j
-  T* vsave;          // the reflectors once more, at j * MR (nullable)
   T* cden;           // [j]: reflector j's coefficient 2/|v|^2 (0: no reflector), with kLate its reciprocal
   T* diag;           // [j]: R_jj
 };
@@ -353,7 +352,6 @@ __device__ __forceinline__ void qr_pivot(T (&x)[QrCfg<T, MR, NC, KR>::CPT][QrCfg
 #pragma unroll
       for (int u = Q::RUN * C0; u < Q::RPT; u += 4) {
         st4(vs + u * G + g * 4, xr + u);
-        if (o.vsave) st4(o.vsave + (size_t)j * MR + u * G + g * 4, xr + u);
       }
       if (g == jr % G) {
         const T den = nrm * (nrm + (x0 >= T(0) ? x0 : -x0));
@@ -441,16 +439,15 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
 
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T* sm = reinterpret_cast<T*>(smem_raw);
-  // CHI = 64 (kBig): M in global scratch, R_c and the previous-row tile read from global
-  // memory where they are stored (the pointers move with the site), shared memory for Y, V
+  // CHI = 64 (kBig): M in global scratch, the previous-row tile read where it is stored (the pointer
+  // moves with the site), shared memory for Y, V and R_c
   constexpr bool kBig = CHI > 32;
-  T* const Rstore_r = args.Rstore + (size_t)real * args.L * D * D;
   // backward-phase layout
   constexpr int DP = JStride<T, CHI>::DP;
   T* Mc = kBig ? args.Mscratch + (size_t)real * D * D : sm;   // D x D col-major, columns j = x*kn + g
   T* Yc = kBig ? sm : Mc + D * D;  // n columns of stride DP (rows >= D zero)
   T* Vc = Yc + D * DP;        // n columns of stride DP (rows >= n zero)
-  T* Rc = kBig ? Rstore_r : Vc + D * DP;   // D x D col-major R_c
+  T* const Rc = Vc + D * DP;  // D x D col-major R_c
   T* Bt = kBig ? nullptr : Rc + D * D;     // previous-row tile [y][al][be]
   // P is written after the SVD (Y is dead by then) and read by the next site's Q = B P before
   // that site's Y is formed; Q is written after this site's V is dead and read before the next
@@ -461,7 +458,7 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
   T* Xs = sm;                 // 2D x D col-major
 
   __shared__ T Wc[8];               // W[x][a][b] at x*4 + a*2 + b
-  int8_t* jv_s = reinterpret_cast<int8_t*>(kBig ? Vc + D * DP : Bt + TILE);   // Jv[r][c], L entries
+  int8_t* jv_s = reinterpret_cast<int8_t*>(kBig ? Rc + D * D : Bt + TILE);   // Jv[r][c], L entries
   int8_t* jh_s = jv_s + args.L;                                // Jh[r+1][c], L-1 entries
   const T eb = (T)exp(beta), ebm = (T)exp(-beta);             // exp(+-beta): every Boltzmann weight
   using QF = QrCfg<T, 2 * D, D, C::RUN>;     // the forward sweep's QR
@@ -545,10 +542,8 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
       }
     };
     // R_0 = [1]
-    if constexpr (kBig) Rc = Rstore;
     for (int e = tid; e < D * D; e += NT) Rc[e] = (e == 0) ? T(1) : T(0);
-    if constexpr (!kBig)
-      for (int e = tid; e < D * D; e += NT) Rstore[e] = (e == 0) ? T(1) : T(0);
+    for (int e = tid; e < D * D; e += NT) Rstore[e] = (e == 0) ? T(1) : T(0);
     // the tile the first sweep starts on: site 0 (forward sweep), frame site L-1 (zip-up)
     if constexpr (!kBig) prefetch_async(Bt, prev + (size_t)(zip ? osite(L - 1) : 0) * TILE, TILE * (int)sizeof(T), tid, NT);
     __syncthreads();
@@ -556,10 +551,7 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
     // ---------------- forward sweep: R factors of the left parts (canonical only) ----------------
     for (int c = 0; !zip && c < L - 1; ++c) {
       set_w(c);
-      if constexpr (kBig) {
-        Rc = Rstore + (size_t)c * D * D;
-        Bt = const_cast<T*>(prev + (size_t)c * TILE);
-      }
+      if constexpr (kBig) Bt = const_cast<T*>(prev + (size_t)c * TILE);
       cp_async_wait_env();
       __syncthreads();
       // X[(x,i),(b,be)] = sum_al (W(x,0,b) R[i][al] + W(x,1,b) R[i][CHI+al]) B[b][al][be]:
@@ -614,7 +606,7 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
         // the reflectors take X's place, column by column of it read by now
         if constexpr (QF::NTQ == 32) __syncwarp();
         else named_barrier<2>(QF::NTQ);
-        const QrOut<T> out{Xs, nullptr, csave, diag};
+        const QrOut<T> out{Xs, csave, diag};
         qr_factor<T, 2 * D, D, C::RUN>(x, D, out, lane, warp, zero_col);
         T mx = 0;
         for (int j = lane; j < D; j += 32)
@@ -630,7 +622,7 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
             for (int u = 0; u < QF::RPT / 2; ++u) {          // rows below D are zero
               const int i = g + QF::G * u;
               const T v = i <= col ? x[q][u] * inv : T(0);
-              if constexpr (!kBig) Rc[col * D + i] = v;      // kBig reads R_{c+1} back from Rstore
+              Rc[col * D + i] = v;
               Rout[col * D + i] = v;
             }
           }
@@ -668,10 +660,7 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
     for (int c = L - 1; c >= 0; --c) {
       // Bt (tile c) and Rc (R_c) were prefetched during the previous site
       set_w(c);
-      if constexpr (kBig) {
-        Rc = Rstore + (size_t)c * D * D;
-        Bt = const_cast<T*>(prev + (size_t)osite(c) * TILE);
-      }
+      if constexpr (kBig) Bt = const_cast<T*>(prev + (size_t)osite(c) * TILE);
       cp_async_wait_env();
       __syncthreads();
       // Q[b][al][g] = sum_be B[b][al][be] P[(b,be)][g]: 4 x 4 register tiles (a mirrored row
@@ -821,8 +810,7 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
         // graded, so it needs fewer sweeps and leaves a smaller tilt in the kept subspace than
         // on Y itself (at L = 256, chi = 32 in FP32: about half the sweeps and a five-fold
         // smaller 99.9th percentile of the conditional error).  Q1 is not kept; Q2's reflectors
-        // overwrite R_c (shared memory, or its slot of the global R store for CHI = 64: R_c is
-        // not read again in this row), their coefficients go to csave.
+        // overwrite R_c, which is not read again in this row, their coefficients go to csave.
         auto none = [](int) { return false; };
         const int g = lane % QB::G, gi = lane / QB::G;
         T x[QB::CPT][QB::RPT];
@@ -837,16 +825,16 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
         };
         if (warp < QB::NTQ / 32) {
           // one body for both; pass 0: Y, its reflectors in Y's place, R1^T to V (stored for the next
-          // pass); pass 1: R1^T, the reflectors in R_c's place (CHI = 64: in V's and saved to R_c),
-          // R2^T to Y, zero outside n x n
+          // pass); pass 1: R1^T, the reflectors in R_c's place, R2^T
+          // to Y, zero outside n x n
 #pragma unroll 1
           for (int pass = 0; pass < 2; ++pass) {
             load(pass ? Vc : Yc);
-            if (pass == 0 || kBig) {                         // the reflectors take the place of what is read
+            if (pass == 0) {                                 // the reflectors take the place of what is read
               if constexpr (QB::NTQ == 32) __syncwarp();
               else named_barrier<2>(QB::NTQ);
             }
-            const QrOut<T> out{pass ? (kBig ? Vc : Rc) : Yc, pass && kBig ? Rc : nullptr, csave, diag};
+            const QrOut<T> out{pass ? Rc : Yc, csave, diag};
             qr_factor<T, D, D, C::RUN>(x, n, out, lane, warp, none);
             T* const to = pass ? Yc : Vc;
 #pragma unroll
@@ -1102,7 +1090,7 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
         }
         __syncthreads();
         // R_{c-1} streams in while the tile and P are formed (the reflectors are consumed)
-        if (!kBig && c > 1) prefetch_async(Rc, Rstore + (size_t)(c - 1) * D * D, D * D * (int)sizeof(T), tid, NT);
+        if (c > 1) prefetch_async(Rc, Rstore + (size_t)(c - 1) * D * D, D * D * (int)sizeof(T), tid, NT);
       }
       // column of the g-th singular vector (already gathered unless zip-up)
       auto vcol = [&](int g) { return zip ? sel[g] : g; };
