@@ -555,24 +555,26 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
       cp_async_wait_env();
       __syncthreads();
       // X[(x,i),(b,be)] = sum_al (W(x,0,b) R[i][al] + W(x,1,b) R[i][CHI+al]) B[b][al][be]:
-      // four (D x CHI) = (D x CHI)(CHI x CHI) products, 4 x 4 register tiles
-      constexpr int TI = D / 4, TB = CHI / 4;
+      // four (D x CHI) = (D x CHI)(CHI x CHI) products in 4 x BW register tiles (BW = 8 where that
+      // still leaves a tile per thread: the combination of R's rows is formed once per tile)
+      constexpr int BW = CHI >= 32 ? 8 : 4, TI = D / 4, TB = CHI / BW;
       for (int u = tid; u < 4 * TI * TB; u += NT) {
         const int xb = u / (TI * TB), rem = u % (TI * TB);
-        const int x = xb >> 1, b = xb & 1, i0 = (rem % TI) * 4, b0 = (rem / TI) * 4;
+        const int x = xb >> 1, b = xb & 1, i0 = (rem % TI) * 4, b0 = (rem / TI) * BW;
         const T w0 = Wc[x * 4 + 0 * 2 + b], w1 = Wc[x * 4 + 1 * 2 + b];
-        T acc[4][4] = {};
-#pragma unroll 4
+        T acc[4][BW] = {};
+#pragma unroll 2
         for (int al = 0; al < CHI; ++al) {
-          T r0[4], r1[4], bv[4];
+          T r0[4], r1[4], bv[BW];
           ld4(Rc + al * D + i0, r0);
           ld4(Rc + (CHI + al) * D + i0, r1);
-          ld4(Bt + b * CHI * CHI + al * CHI + b0, bv);
+#pragma unroll
+          for (int jj = 0; jj < BW; jj += 4) ld4(Bt + b * CHI * CHI + al * CHI + b0 + jj, bv + jj);
 #pragma unroll
           for (int ii = 0; ii < 4; ++ii) {
             const T rw = w0 * r0[ii] + w1 * r1[ii];
 #pragma unroll
-            for (int jj = 0; jj < 4; ++jj) acc[ii][jj] += rw * bv[jj];
+            for (int jj = 0; jj < BW; ++jj) acc[ii][jj] += rw * bv[jj];
           }
         }
         // row (x, i) of X is stored at 2 i + x: the two blocks R_c A^0 and R_c A^1 share
@@ -580,7 +582,7 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
         // the rows in order of scale (measured at L = 256 in FP32: two orders of magnitude
         // fewer clamped weights than the two blocks one after the other)
 #pragma unroll
-        for (int jj = 0; jj < 4; ++jj) {
+        for (int jj = 0; jj < BW; ++jj) {
           T* xc = Xs + (size_t)(b * CHI + b0 + jj) * (2 * D);
 #pragma unroll
           for (int ii = 0; ii < 4; ++ii) xc[qr_pos<QF::G>(2 * (i0 + ii) + x)] = acc[ii][jj];
