@@ -86,7 +86,8 @@ constexpr int kThreadStages = 4;      // environment tiles in flight per warp
 // are left out, which at L = 8, chi = 16 is five sixths of the products.
 // What bounds it: in FP64 the FP64 pipe (a warp's multiply-add takes 64 of a scheduler's cycles), which a
 // lane per bond index left half empty at chi = 16 and busy with every proposal's logarithm and divisions
-// 32 times over; in FP32 the chain of one site after the other.  One GB300, propose(): L = 8, chi = 16,
+// 32 times over; in FP32 the chain of one site after the other (few proposals, up to four CTAs of
+// sample_kernel per SM, are sample_kernel's).  One GB300, propose(): L = 8, chi = 16,
 // 100 x 1000 proposals in FP64 62 -> 9.7 ms; L = 16, chi = 8, 64 x 400 in FP32 4.2 -> 0.77 ms.
 template <typename T, typename TE, int CHI>
 __global__ void __launch_bounds__(128, kThreadWarps / 4)
@@ -786,12 +787,22 @@ template <typename T, typename TE, int CHI>
 static cudaError_t launch_sample_t(const SampleArgs& a, int num_sms, cudaStream_t st) {
   constexpr int NW = kSampleWarps;
   if constexpr (CHI <= 16) {
-    // One thread per proposal, in FP64 from CHI^2 / 8 proposals per SM on: below that too few warps
-    // share the FP64 pipes and one thread's chain over the bond index is what the call waits for
-    // (L = 24, chi = 16: 27 ms for any number up to 19456 against 7.0 ms per 1216 of the other kernel,
-    // equal at 4096; chi = 8, L = 12: equal at about 1300; chi = 4, L = 16: at about 300).
-    if (sizeof(T) == 4 || (int64_t)a.n_items * a.n_real >= (int64_t)num_sms * (CHI * CHI / 8))
-      return launch_sample_thread<T, TE, CHI>(a, num_sms, st);
+    // One thread per proposal from a number of proposals on; below it, too few warps are in flight and
+    // one thread's chain over the bond index is what the call waits for.  Its time is the same for any
+    // number that the slots hold at once, that of the other kernel goes by the CTAs (NW proposals of a
+    // realization each) that an SM gets.  propose() at L = 16, one GB300, ms of this kernel (first) and
+    // of the other one at 1, 2 and 4 CTAs per SM:
+    //   FP32 chi = 4  0.39 | 0.40 0.49 0.75     FP64 chi = 4   2.7 | 2.5 4.8  9.6
+    //   FP32 chi = 8  0.67 | 0.42 0.49 0.79     FP64 chi = 8   4.9 | 2.7 5.2 13.0
+    //   FP32 chi = 16 1.40 | 0.47 0.59 1.00     FP64 chi = 16 10.8 | 3.1 6.0 15.1
+    // (BF16 as FP32; beyond 4 the other kernel's grow in proportion).  The line is drawn where this
+    // kernel is the faster one in propose() and in eval_conditionals().  With more tiles than slots
+    // (large L) each further pass over the slots costs as much again.
+    constexpr int kLimit = sizeof(T) == 4 ? (CHI == 4 ? 1 : 4) : (CHI == 16 ? 3 : 1);
+    const int64_t ctas = (int64_t)((a.n_items + NW - 1) / NW) * a.n_real;
+    const int64_t tiles = (int64_t)((a.n_items + 31) / 32) * a.n_real, slots = thread_slots<T>(a.L, CHI, num_sms);
+    const int64_t passes = (tiles + slots - 1) / slots;
+    if (ctas > (passes > 1 ? 4 * passes : kLimit) * num_sms) return launch_sample_thread<T, TE, CHI>(a, num_sms, st);
   }
   const size_t smem = sample_smem<CHI, NW>(a.L, sizeof(TE));
   void (*kern)(SampleArgs);

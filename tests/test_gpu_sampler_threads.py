@@ -64,3 +64,16 @@ def test_conditionals_against_oracle(tn, L, chi, n, precision):
         assert np.array_equal(energy[k].reshape(2 * n)[:3].numpy(), lattice.energy(s, Jh, Jv))
         m = min(3, n)                                    # the first chain's proposals among them
         assert torch.equal(lq[k][:m], logq[k].reshape(2 * n)[:m])
+
+
+# The same in FP32 and BF16: more than four CTAs of eight proposals per SM take the thread's path, in
+# whole tiles of 32 and in tiles that a realization's proposals do not fill.
+@pytest.mark.parametrize("L,chi,crowd,n", [(3, 2, 700, 5), (8, 4, 160, 33), (9, 7, 700, 5), (12, 8, 160, 33),
+                                           (11, 13, 160, 33), (16, 16, 1300, 1)])
+@pytest.mark.parametrize("precision", ["fp32", "bf16"])
+def test_fp32_same_bits_alone_and_in_a_crowd(tn, L, chi, crowd, n, precision):
+    seeds = list(range(40, 40 + crowd))
+    many = _run(tn, L, chi, seeds, n, precision)
+    few = _run(tn, L, chi, seeds[:2], n, precision)
+    for a, b in zip(many, few):
+        assert torch.equal(a[:2], b)
