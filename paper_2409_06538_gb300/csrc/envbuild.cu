@@ -86,16 +86,16 @@ __device__ __forceinline__ void rot16(double2& u, double2& v, double c, double s
 //   s = sgn(b-a) g / (r c)   (sgn(0) = +1),
 // two reciprocal square roots in sequence instead of the divide/sqrt chain of the tangent
 // form.  FP32 uses the hardware rsqrt with one Newton step each, so c^2 + s^2 = 1 to
-// working precision; FP64 uses IEEE operations.
+// working precision; FP64 calls the library's, which leaves out a root and a division each.
 __device__ __forceinline__ float rsqrt_nr(float x) {
   const float r = rsqrtf(x);
   return r * fmaf(-0.5f * x * r, r, 1.5f);
 }
 __device__ __forceinline__ void rotation_from_gram(double a, double b, double g, double& c, double& s) {
   const double d = b - a;
-  const double rinv = 1.0 / sqrt(d * d + 4.0 * g * g);
-  const double h = 0.5 + 0.5 * fabs(d) * rinv;
-  const double ic = 1.0 / sqrt(h);
+  const double rinv = rsqrt(fma(d, d, 4.0 * g * g));
+  const double h = fma(0.5 * fabs(d), rinv, 0.5);
+  const double ic = rsqrt(h);
   c = h * ic;
   s = (d < 0.0 ? -g : g) * rinv * ic;
 }
@@ -203,13 +203,20 @@ __host__ __device__ constexpr size_t env_smem_elems() {
 // shuffles (30 cycles a level).  Environment build at chi = 32, FP32 (one GB300): 203 -> 150 us a site
 // step with one realization per SM (L = 64), 331 -> 214 us with three (L = 48).
 template <typename T, int MR, int NC, int KR> struct QrCfg {
-  static constexpr int G = MR >= 32 ? MR / 16 : 2;          // lanes of a column: 16 rows each from MR = 32 on
+  // Lanes of a column: 16 rows each from MR = 32 on.  FP64 to MR = 32: four rows each, as an operation
+  // of a warp keeps a scheduler's FP64 pipe for 64 cycles, so that a chain of few rows is the shorter
+  // one (at MR = 64 the threads that this takes make it the longer one).  FP64 build with the roots of
+  // norm_of and rotation_from_gram, before and after: chi = 16, L = 24, 256 realizations 404 -> 363 ms;
+  // chi = 8, L = 12, 608 of them 28.5 -> 23.9 ms; chi = 32, L = 12, 8 of them 82.1 -> 78.4 ms (at 16
+  // rows a lane as here; 89.8 ms with four).
+  static constexpr bool FEW = sizeof(T) == 8 && MR <= 32;
+  static constexpr int G = FEW ? (MR >= 8 ? MR / 4 : 2) : (MR >= 32 ? MR / 16 : 2);
   static constexpr int RPT = MR / G;
-  static constexpr int NVL = 32 / G < RPT ? 32 / G : RPT;   // partial sums a lane holds
+  static constexpr int NVL = 32 / G < RPT ? 32 / G : RPT;   // partial sums a lane holds (not if FEW)
   // The factorisation has one body for each run of KR rows of a lane (the pivots whose rows are in
   // it; the rows of earlier runs are left out): short runs save products of zeros and cost code.
   static constexpr int RUN = RPT < KR ? RPT : KR;
-  static constexpr int CPT = NC * G > 512 ? (NC * G) / 512 : (NC * G > 256 ? 2 : 1);
+  static constexpr int CPT = NC * G > 512 ? (NC * G) / 512 : (NC * G > 256 || G > 4 ? 2 : 1);
   static constexpr int NTQ = NC * G / CPT < 32 ? 32 : NC * G / CPT;   // threads taking part
   static constexpr int GPW = 32 / G;                        // groups of a warp
   static constexpr int CW = GPW * CPT;                      // columns of a warp
@@ -251,26 +258,41 @@ __device__ __forceinline__ void add_pair(double* p, const double* q) { p[0] += q
 // Sum of v * x over the rows of the runs C0 and later (the earlier ones hold zeros) in the fixed
 // association; every lane of the group gets it.
 template <typename Q, int C0, typename T>
-__device__ __forceinline__ T qr_dot(const T (&v)[Q::RPT], const T (&x)[Q::RPT]) {
-  T p[Q::NVL];
+__device__ __forceinline__ T qr_dot(const T (&v)[Q::RPT], const T (&x)[Q::RPT], int j) {
+  T d;
+  if constexpr (Q::FEW) {
+    // one chain; rows above the pivot j hold zeros in v
+    d = T(0);
 #pragma unroll
-  for (int a = 0; a < Q::NVL; ++a) p[a] = T(0);
+    for (int u = 0; u < Q::RPT; ++u)
+      if (Q::G * (u + 1) > j) d = fma(v[u], x[u], d);
+  } else {
+    T p[Q::NVL];
 #pragma unroll
-  for (int u = Q::RUN * C0; u < Q::RPT; u += 2) fma_pair(v + u, x + u, p + u % Q::NVL);
+    for (int a = 0; a < Q::NVL; ++a) p[a] = T(0);
 #pragma unroll
-  for (int lv = Q::NVL / 2; lv > 1; lv >>= 1)
+    for (int u = Q::RUN * C0; u < Q::RPT; u += 2) fma_pair(v + u, x + u, p + u % Q::NVL);
 #pragma unroll
-    for (int a = 0; a < lv; a += 2) add_pair(p + a, p + a + lv);
-  T d = p[0] + p[1];
+    for (int lv = Q::NVL / 2; lv > 1; lv >>= 1)
+#pragma unroll
+      for (int a = 0; a < lv; a += 2) add_pair(p + a, p + a + lv);
+    d = p[0] + p[1];
+  }
 #pragma unroll
   for (int o = Q::G / 2; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
   return d;
 }
 template <typename Q, int C0, typename T>
-__device__ __forceinline__ void qr_update(T md, const T (&v)[Q::RPT], T (&x)[Q::RPT]) {
-  const T m2[2] = {md, md};
+__device__ __forceinline__ void qr_update(T md, const T (&v)[Q::RPT], T (&x)[Q::RPT], int j) {
+  if constexpr (Q::FEW) {
 #pragma unroll
-  for (int u = Q::RUN * C0; u < Q::RPT; u += 2) fma_pair(m2, v + u, x + u);
+    for (int u = 0; u < Q::RPT; ++u)
+      if (Q::G * (u + 1) > j) x[u] = fma(md, v[u], x[u]);
+  } else {
+    const T m2[2] = {md, md};
+#pragma unroll
+    for (int u = Q::RUN * C0; u < Q::RPT; u += 2) fma_pair(m2, v + u, x + u);
+  }
 }
 template <typename Q, int C0, typename T>
 __device__ __forceinline__ void qr_load_v(const T* vs, int g, T (&v)[Q::RPT]) {
@@ -320,6 +342,15 @@ __device__ __forceinline__ float inverse(float x) {
 }
 __device__ __forceinline__ double inverse(double x) { return 1.0 / x; }
 
+// Square root of a column's squared norm.  In FP64 from the reciprocal root and one step of Newton's
+// iteration, s + (ss - s^2) / (2 s): half the instructions of the pipe that the factorisation waits for.
+__device__ __forceinline__ float norm_of(float ss) { return sqrtf(ss); }
+__device__ __forceinline__ double norm_of(double ss) {
+  if (!(ss > 0.0 && ss < INFINITY)) return ss;
+  const double r = rsqrt(ss), s = ss * r;
+  return fma(0.5 * r, fma(-s, s, ss), s);
+}
+
 // Reflector of column j, by the warp that owns it; j lies in the rows of run C0.
 template <typename T, int MR, int NC, int KR, int C0>
 __device__ __forceinline__ void qr_pivot(T (&x)[QrCfg<T, MR, NC, KR>::CPT][QrCfg<T, MR, NC, KR>::RPT], int j, T* vs,
@@ -340,9 +371,9 @@ __device__ __forceinline__ void qr_pivot(T (&x)[QrCfg<T, MR, NC, KR>::CPT][QrCfg
       if (i < jr) xr[Q::RUN * C0 + u] = T(0);
       if (i == jr) x0 = xr[Q::RUN * C0 + u];
     }
-    const T ss = qr_dot<Q, C0, T>(xr, xr);
+    const T ss = qr_dot<Q, C0, T>(xr, xr, j);
     const bool null = ss <= tiny;
-    const T nrm = num<T>::sqrt_(ss);
+    const T nrm = norm_of(ss);
     if (gi == jl - jq * Q::GPW) {            // the pivot's group
       const T alpha = x0 >= T(0) ? -nrm : nrm;
       const T v0 = x0 - alpha;
@@ -389,9 +420,9 @@ __device__ __forceinline__ void qr_runs(T (&x)[QrCfg<T, MR, NC, KR>::CPT][QrCfg<
         const T coef = !kLate<T> || den == T(0) ? den : inverse(den);
 #pragma unroll
         for (int q = 0; q < Q::CPT; ++q) {
-          T d = qr_dot<Q, C0, T>(v, x[q]) * coef;
+          T d = qr_dot<Q, C0, T>(v, x[q], j) * coef;
           if (first + q * Q::GPW + gi <= j) d = T(0);
-          qr_update<Q, C0>(-d, v, x[q]);
+          qr_update<Q, C0>(-d, v, x[q], j);
         }
       }
     }
@@ -420,8 +451,8 @@ __device__ __forceinline__ void qr_apply_q(T (&x)[QrCfg<T, MR, NC, KR>::RPT], in
     if (coef == T(0)) continue;
     T v[Q::RPT];
     qr_load_v<Q, C0, T>(vs + (size_t)j * MR, g, v);
-    const T d = qr_dot<Q, C0, T>(v, x) * coef;
-    qr_update<Q, C0>(-d, v, x);
+    const T d = qr_dot<Q, C0, T>(v, x, j) * coef;
+    qr_update<Q, C0>(-d, v, x, j);
   }
   if constexpr (C0 > 0) qr_apply_q<T, MR, NC, KR, C0 - 1>(x, n, vs, coefs, g);
 }
