@@ -25,6 +25,7 @@
 // bonds swapped, horizontal bond factors at the bond's right site).
 #include "common.cuh"
 #include "kernels.h"
+#include "rounding.cuh"
 
 namespace tnmc {
 
@@ -332,15 +333,22 @@ template <typename T> struct QrOut {
 // where a division occupies the FP64 pipe, only the pivot's warp does.
 template <typename T> constexpr bool kLate = sizeof(T) == 4;
 
-// 1 / x, correctly rounded for normal x and 1 / x: the hardware's approximation and one Newton step with
-// a fused residual (Markstein 1990), checked against the division for every float in [1e-37, 1e37].
-// The division's branch for its special cases keeps it from overlapping with the dot products.
-__device__ __forceinline__ float inverse(float x) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return fmaf(r, fmaf(-x, r, 1.0f), r);
+// The range of inverse() ends at a coefficient of 8e37, at most twice a column's squared norm.  A matrix that
+// may go beyond it (weights of exp(36) and more: strong fields, low temperatures) is factored times kDown, a
+// power of two, so nothing is rounded by it; nothing has to be scaled back either, as R is normalised, the
+// right singular vectors have no scale and the singular values are only compared.  One that is too large for
+// that as well becomes NaN, which the sampler flags.  Whoever forms a matrix looks at its entries, and the
+// scaling is out of line: that costs 1 % of the builds for chi <= 8, 4 % of the crowd's, whose code is the
+// tightest (90.5 -> 93.9 ms, 1024 realizations of 32 x 32), and nothing beyond.  A test of each coefficient in
+// the warps that use it cost 2 to 4 % of all, in the pivot's warp 3 to 8 %, a second body that divides 1 to 3 %.
+constexpr float kLargeEntry = 1e16f;                 // 2 * 128 * 128 entries * kLargeEntry^2 = 3.3e36
+constexpr float kDown = 1.0f / 4294967296.0f;        // 2^-32
+__device__ __forceinline__ float entry_max(float m, float x) { return fmaxf(m, fabsf(x)); }
+__device__ __forceinline__ double entry_max(double m, double) { return m; }
+// What an entry makes of its matrix: 0, 1 beyond kLargeEntry, 2 beyond what kDown brings back.
+template <typename T> __device__ __forceinline__ void note_large(T entry, int* flag) {
+  if (kLate<T> && entry > T(kLargeEntry)) atomicMax(flag, entry * T(kDown) > T(kLargeEntry) ? 2 : 1);
 }
-__device__ __forceinline__ double inverse(double x) { return 1.0 / x; }
 
 // Square root of a column's squared norm.  In FP64 from the reciprocal root and one step of Newton's
 // iteration, s + (ss - s^2) / (2 s): half the instructions of the pipe that the factorisation waits for.
@@ -457,6 +465,18 @@ __device__ __forceinline__ void qr_apply_q(T (&x)[QrCfg<T, MR, NC, KR>::RPT], in
   if constexpr (C0 > 0) qr_apply_q<T, MR, NC, KR, C0 - 1>(x, n, vs, coefs, g);
 }
 
+// a[c][i] (i < rows, columns ld apart) times s; returns the sum of squares of the thread's own entries.
+template <typename T> __device__ __noinline__ T scale_matrix(T* a, int rows, int cols, int ld, T s, int tid, int nt) {
+  T f = 0;
+#pragma unroll 1
+  for (int e = tid; e < rows * cols; e += nt) {
+    T& y = a[(size_t)(e / rows) * ld + e % rows];
+    y *= s;
+    f += y * y;
+  }
+  return f;
+}
+
 template <typename T, typename TE, int CHI, bool kCrowd>
 __global__ void __launch_bounds__(EnvCfg<CHI>::NT, sizeof(T) == 8 ? 1 : EnvCfg<CHI, kCrowd>::PER_SM)
 env_build_kernel(EnvBuildArgs<T, TE> args) {
@@ -501,6 +521,7 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
   __shared__ int sel[CHI];
   __shared__ int rot[3];            // per-sweep 'any rotation' flags, a ring of three
   __shared__ int knext_s;
+  __shared__ int large_s;           // of the matrix to be factored, as note_large leaves it
 
   const int8_t* J = args.J + (size_t)real * 2 * L * (L - 1);
   // external fields (units of beta) of this realization: the row MPO carries those of the row
@@ -582,6 +603,7 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
     // ---------------- forward sweep: R factors of the left parts (canonical only) ----------------
     for (int c = 0; !zip && c < L - 1; ++c) {
       set_w(c);
+      if (tid == 0) large_s = 0;
       if constexpr (kBig) Bt = const_cast<T*>(prev + (size_t)c * TILE);
       cp_async_wait_env();
       __syncthreads();
@@ -589,6 +611,7 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
       // four (D x CHI) = (D x CHI)(CHI x CHI) products in 4 x BW register tiles (BW = 8 where that
       // still leaves a tile per thread: the combination of R's rows is formed once per tile)
       constexpr int BW = CHI >= 32 ? 8 : 4, TI = D / 4, TB = CHI / BW;
+      T xmax = 0;
       for (int u = tid; u < 4 * TI * TB; u += NT) {
         const int xb = u / (TI * TB), rem = u % (TI * TB);
         const int x = xb >> 1, b = xb & 1, i0 = (rem % TI) * 4, b0 = (rem / TI) * BW;
@@ -616,10 +639,19 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
         for (int jj = 0; jj < BW; ++jj) {
           T* xc = Xs + (size_t)(b * CHI + b0 + jj) * (2 * D);
 #pragma unroll
-          for (int ii = 0; ii < 4; ++ii) xc[qr_pos<QF::G>(2 * (i0 + ii) + x)] = acc[ii][jj];
+          for (int ii = 0; ii < 4; ++ii) {
+            xc[qr_pos<QF::G>(2 * (i0 + ii) + x)] = acc[ii][jj];
+            xmax = entry_max(xmax, acc[ii][jj]);
+          }
         }
       }
+      note_large(xmax, &large_s);
       __syncthreads();
+      if (kLate<T> && large_s) {
+        const T s = large_s > 1 ? T(NAN) : T(kDown);
+        scale_matrix<T>(Xs, 2 * D, D, 2 * D, s, tid, NT);
+        __syncthreads();
+      }
       // the next site's tile streams in while the QR runs
       if constexpr (!kBig) prefetch_async(Bt, prev + (size_t)(c + 1) * TILE, TILE * (int)sizeof(T), tid, NT);
       // R factor of X in registers; R_{c+1} = R / max |R_jj| (col-major, zeros below the diagonal)
@@ -693,6 +725,7 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
     for (int c = L - 1; c >= 0; --c) {
       // Bt (tile c) and Rc (R_c) were prefetched during the previous site
       set_w(c);
+      if (tid == 0) large_s = 0;
       if constexpr (kBig) Bt = const_cast<T*>(prev + (size_t)osite(c) * TILE);
       cp_async_wait_env();
       __syncthreads();
@@ -786,6 +819,7 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
       } else {
         constexpr int TI = D / 4;
         const int TJ = (n + 3) / 4;
+        T ymax = 0;
         for (int u = tid; u < TI * TJ; u += NT) {
           const int i0 = (u % TI) * 4, j0 = (u / TI) * 4;
           T acc[4][4] = {};
@@ -812,12 +846,14 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
 #pragma unroll
               for (int ii = 0; ii < 4; ++ii) {
                 Yc[(size_t)(j0 + jj) * DP + qr_pos<QB::G>(i0 + ii)] = acc[ii][jj];
+                ymax = entry_max(ymax, acc[ii][jj]);
 #pragma unroll
                 for (int q = 0; q < VK; ++q) if ((u / NT) % VK == q) fro[q] += acc[ii][jj] * acc[ii][jj];
               }
             }
           }
         }
+        note_large(ymax, &large_s);
       }
       // the Jacobi runs on npad = n rounded up to 8 columns (blocks of 4, an even number of
       // blocks); columns n..npad-1 of Y are zero and never rotate
@@ -829,7 +865,17 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
       }
       if (tid == 0) { rot[0] = 0; rot[1] = 0; rot[2] = 0; }
       __syncthreads();
-      const T tinyY = warp_sum(lane < C::VT / 32 ? red[lane] : T(0)) * num<T>::eps * num<T>::eps;
+      T sumY = warp_sum(lane < C::VT / 32 ? red[lane] : T(0));
+      if (kLate<T> && large_s) {             // (never set in zip-up mode)
+        const T s = large_s > 1 ? T(NAN) : T(kDown);
+        T f = scale_matrix<T>(Yc, D, n, DP, s, tid, NT);
+        f = warp_sum(f);
+        __syncthreads();
+        if (lane == 0) red[warp] = f;
+        __syncthreads();
+        sumY = warp_sum(lane < NWARP ? red[lane] : T(0));
+      }
+      const T tinyY = sumY * num<T>::eps * num<T>::eps;
       if (zip) {
         // the zip-up's Y = M is graded by columns (P = U S), where the one-sided Jacobi is
         // accurate without preconditioning

@@ -35,6 +35,7 @@
 // L = 48, 448 x 500 158 -> 65 ms; CHI = 16, L = 32, 1024 x 2000 246 -> 140 ms.
 #include "common.cuh"
 #include "kernels.h"
+#include "rounding.cuh"
 
 namespace tnmc {
 namespace tc {
@@ -121,23 +122,11 @@ __device__ __forceinline__ void tmem_st8(uint32_t ta, const float* v) {
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// The same rounding of a finite x below the largest binade, in two integer operations: half of
-// the 11-bit significand's last place is added to the magnitude and the rest cut off (checked against
-// the instruction for every such float).  cvt.rna takes four issue slots.
-__device__ __forceinline__ float tf32_rna_finite(float x) {
-  return __uint_as_float((__float_as_uint(x) + 0x1000u) & 0xffffe000u);
-}
 __device__ __forceinline__ float max_nan(float a, float b) {       // NaN if either is
   float r;
   asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
   return r;
 }
-__device__ __forceinline__ float tf32_rna(float x) {
-  uint32_t r;
-  asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-  return __uint_as_float(r);
-}
-
 // Float offset of element (row r, k) in a (rows x KD) K-major canonical operand.
 template <int KD> __device__ __forceinline__ int koff(int r, int k) {
   return (r >> 3) * (8 * KD) + (k >> 2) * 32 + (r & 7) * 4 + (k & 3);
