@@ -1335,8 +1335,7 @@ template <typename T, typename TE, int CHI, bool kCrowd>
 static cudaError_t env_build_setup(int L, size_t* smem) {
   // + the two rows' couplings (int8) staged behind the tile
   *smem = env_smem_elems<T, CHI>() * sizeof(T) + (size_t)2 * L + 16;
-  return cudaFuncSetAttribute(env_build_kernel<T, TE, CHI, kCrowd>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)*smem);
+  return allow_shared_memory<env_build_kernel<T, TE, CHI, kCrowd>>();
 }
 
 template <typename T, typename TE, int CHI, bool kCrowd = false>

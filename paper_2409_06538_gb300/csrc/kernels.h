@@ -5,7 +5,29 @@
 #include <stdint.h>
 #include <stddef.h>
 
+#include <atomic>
+
 namespace tnmc {
+
+// Lets Kern be launched with as much dynamic shared memory as a block can have on the current device.  The
+// limit belongs to the kernel, not to a launch: raised once and never lowered, since contexts of other sizes
+// may be launching the same kernel from other threads.
+template <auto Kern>
+cudaError_t allow_shared_memory() {
+  static std::atomic<uint64_t> done{0};          // a bit per device
+  int dev = 0, optin = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const uint64_t bit = dev < 64 ? (uint64_t)1 << dev : 0;
+  if (done.load(std::memory_order_acquire) & bit) return cudaSuccess;
+  cudaFuncAttributes fa;
+  e = cudaFuncGetAttributes(&fa, Kern);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(Kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
+  if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_release);
+  return e;
+}
 
 // Device status bits (OR-ed into the context's status word).
 enum : unsigned {

@@ -773,8 +773,7 @@ template <typename T, typename TE, int CHI>
 static cudaError_t launch_sample_thread(const SampleArgs& a, int num_sms, cudaStream_t st) {
   const size_t smem = 4 * ((size_t)kThreadStages * 2 * CHI * CHI * sizeof(TE) + 2 * (size_t)((a.L + 15) & ~15) +
                            (size_t)((a.L + 31) / 32) * 128);
-  cudaError_t e = cudaFuncSetAttribute(sample_thread_kernel<T, TE, CHI>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
+  cudaError_t e = allow_shared_memory<sample_thread_kernel<T, TE, CHI>>();
   if (e != cudaSuccess) return e;
   const int64_t tiles = (int64_t)((a.n_items + 31) / 32) * a.n_real;
   int64_t slots = thread_slots<T>(a.L, CHI, num_sms);
@@ -805,10 +804,11 @@ static cudaError_t launch_sample_t(const SampleArgs& a, int num_sms, cudaStream_
     if (ctas > (passes > 1 ? 4 * passes : kLimit) * num_sms) return launch_sample_thread<T, TE, CHI>(a, num_sms, st);
   }
   const size_t smem = sample_smem<CHI, NW>(a.L, sizeof(TE));
-  void (*kern)(SampleArgs);
-  if constexpr (CHI > 32) kern = sample_kernel_wide<T, TE, CHI, NW>;
-  else kern = sample_kernel<T, TE, CHI, NW>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  constexpr auto kern = [] {
+    if constexpr (CHI > 32) return &sample_kernel_wide<T, TE, CHI, NW>;
+    else return &sample_kernel<T, TE, CHI, NW>;
+  }();
+  cudaError_t e = allow_shared_memory<kern>();
   if (e != cudaSuccess) return e;
   int per_sm = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 32 * NW, smem);

@@ -654,19 +654,15 @@ static cudaError_t launch_tc_t(const SampleArgs& a, int num_sms, cudaStream_t st
     if (sample_tc_grid(a.n_items, a.n_real, CHI, num_sms) <= 2 * num_sms) return launch_tc_t<CHI, 2>(a, num_sms, st);
   // Three raw tiles in flight where PER_SM CTAs still fit on an SM (CHI = 32: L up to about 210), else
   // two: at L = 256 a second CTA is worth more than the third tile.
+  const cudaError_t e = allow_shared_memory<sample_tc_kernel<CHI, PER_SM>>();
+  if (e != cudaSuccess) return e;
   int raw_tiles = 3, fit = 0;
   size_t smem = 0;
   for (;; --raw_tiles) {
     smem = sample_tc_smem<CHI>(a.L, raw_tiles);
-    cudaError_t e = cudaFuncSetAttribute(sample_tc_kernel<CHI, PER_SM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e == cudaSuccess)
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, sample_tc_kernel<CHI, PER_SM>, tc::Cfg<CHI>::NT, smem);
-    if (e == cudaSuccess && fit >= PER_SM) break;
-    if (raw_tiles == 2) {
-      if (e != cudaSuccess) return e;
-      break;
-    }
-    cudaGetLastError();
+    const cudaError_t q = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, sample_tc_kernel<CHI, PER_SM>, tc::Cfg<CHI>::NT, smem);
+    if (q != cudaSuccess) cudaGetLastError();
+    if (raw_tiles == 2 || (q == cudaSuccess && fit >= PER_SM)) break;
   }
   const int grid = sample_tc_grid(a.n_items, a.n_real, CHI, num_sms);
   sample_tc_kernel<CHI, PER_SM><<<grid, tc::Cfg<CHI>::NT, smem, st>>>(a, raw_tiles);
