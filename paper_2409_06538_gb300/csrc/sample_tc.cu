@@ -176,7 +176,8 @@ template <int CHI> struct Cfg {
   static constexpr int TILE = 2 * BOP;              // floats of one cached site tile [y][al][be]
   static constexpr int STAGE = 4 * BOP;             // [hi y0, hi y1, lo y0, lo y1]
   static constexpr int NST = CHI <= 16 ? 4 : 3;     // stages
-  static constexpr int RAWTILE = 2 * CHI * (CHI + 4);
+  // tiles as they are in global memory: one being split, one on its way (a third was no faster at any size)
+  static constexpr int RAWTILE = 2 * CHI * (CHI + 4), NRAW = 2;
   // tensor memory: accumulators of y = 0, 1, then the A rows R0 (or l) hi, lo, R1 hi, lo
   static constexpr int TCOLS = 6 * CHI <= 128 ? 128 : 256;
   // CTAs per SM: tensor memory and registers allow two at CHI = 32, three at 16
@@ -186,7 +187,7 @@ template <int CHI> struct Cfg {
 }  // namespace tc
 
 template <int CHI, int PER_SM>
-__global__ void __launch_bounds__(tc::Cfg<CHI>::NT, PER_SM) sample_tc_kernel(SampleArgs a, int raw_tiles) {
+__global__ void __launch_bounds__(tc::Cfg<CHI>::NT, PER_SM) sample_tc_kernel(SampleArgs a) {
   using namespace tc;
   using C = Cfg<CHI>;
   constexpr int BOP = C::BOP, TILE = C::TILE, NST = C::NST;
@@ -198,7 +199,7 @@ __global__ void __launch_bounds__(tc::Cfg<CHI>::NT, PER_SM) sample_tc_kernel(Sam
   float* Bbuf = smf;                                  // [stage][hi y0, hi y1, lo y0, lo y1]
   const int LP = (L + 15) & ~15;                      // keeps the uint32 arrays 16-byte aligned
   float* Rawbuf = Bbuf + NST * C::STAGE;              // [buffer][y, al][be], rows padded
-  float* Rws = Rawbuf + raw_tiles * C::RAWTILE;          // [y][j / 4][proposal][4]
+  float* Rws = Rawbuf + C::NRAW * C::RAWTILE;         // [y][j / 4][proposal][4]
   int8_t* jrow = reinterpret_cast<int8_t*>(Rws + 2 * CHI * M);      // [proposal warp][Jh row, Jv row above]
   uint32_t* prow = reinterpret_cast<uint32_t*>(jrow + 8 * LP);          // [words_row][M]
   __shared__ __align__(8) uint64_t bar_a, bar_d, bar_full[NST], bar_free[NST];
@@ -255,12 +256,12 @@ __global__ void __launch_bounds__(tc::Cfg<CHI>::NT, PER_SM) sample_tc_kernel(Sam
           const uint32_t d = su32(dst + (u / (CHI / 4)) * RS + 4 * (u % (CHI / 4)));
           asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(tile + 4 * u) : "memory");
         }
-        lb = lb + 1 == raw_tiles ? 0 : lb + 1;
+        lb ^= 1;
         if (++li == 2 * L - 1) { li = 0; if (++lr == L) { lr = 0; lt += gridDim.x; } }
       }
       asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    for (int d = 0; d < raw_tiles - 1; ++d) copy_next();
+    copy_next();
     const int64_t mine = blockIdx.x < total ? (total - 1 - blockIdx.x) / gridDim.x + 1 : 0;
     const int64_t operands = mine * L * (2 * L - 1);
     int i = 0, rb = 0, st = 0;
@@ -268,8 +269,7 @@ __global__ void __launch_bounds__(tc::Cfg<CHI>::NT, PER_SM) sample_tc_kernel(Sam
     for (int64_t n = 0; n < operands; ++n) {
       // this tile's copy has arrived and the stage is free, for every tile warp; all are done with
       // the raw tile before this one, whose buffer takes the next copy
-      if (raw_tiles > 2) asm volatile("cp.async.wait_group 1;" ::: "memory");
-      else asm volatile("cp.async.wait_group 0;" ::: "memory");
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
       const bool ok = round == 0 || wait_or_abort(&bar_free[st], (round - 1) & 1u);
       if (any_of<C::NPROD>(1, !ok)) break;            // all of them leave, or none
       copy_next();
@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(tc::Cfg<CHI>::NT, PER_SM) sample_tc_kernel(Sam
       __syncwarp();
       if ((tid & 31) == 0) mbar_arrive(&bar_full[st]);
       if (++i == 2 * L - 1) i = 0;
-      rb = rb + 1 == raw_tiles ? 0 : rb + 1;
+      rb ^= 1;
       if (++st == NST) { st = 0; ++round; }
     }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
@@ -626,10 +626,10 @@ __global__ void __launch_bounds__(tc::Cfg<CHI>::NT, PER_SM) sample_tc_kernel(Sam
 }
 
 template <int CHI>
-static size_t sample_tc_smem(int L, int raw_tiles) {
+static size_t sample_tc_smem(int L) {
   using C = tc::Cfg<CHI>;
   const int words_row = (L + 31) / 32;
-  return (size_t)(C::NST * C::STAGE + raw_tiles * C::RAWTILE + 2 * CHI * tc::M) * sizeof(float) +
+  return (size_t)(C::NST * C::STAGE + C::NRAW * C::RAWTILE + 2 * CHI * tc::M) * sizeof(float) +
          (size_t)8 * ((L + 15) & ~15) + (size_t)words_row * tc::M * sizeof(uint32_t) + 64;
 }
 
@@ -652,20 +652,10 @@ static cudaError_t launch_tc_t(const SampleArgs& a, int num_sms, cudaStream_t st
   // 2.8 -> 2.6 ms, while 16384 tiles take 158 ms with two CTAs per SM against 140 with three).
   if constexpr (PER_SM > 2)
     if (sample_tc_grid(a.n_items, a.n_real, CHI, num_sms) <= 2 * num_sms) return launch_tc_t<CHI, 2>(a, num_sms, st);
-  // Three raw tiles in flight where PER_SM CTAs still fit on an SM (CHI = 32: L up to about 210), else
-  // two: at L = 256 a second CTA is worth more than the third tile.
   const cudaError_t e = allow_shared_memory<sample_tc_kernel<CHI, PER_SM>>();
   if (e != cudaSuccess) return e;
-  int raw_tiles = 3, fit = 0;
-  size_t smem = 0;
-  for (;; --raw_tiles) {
-    smem = sample_tc_smem<CHI>(a.L, raw_tiles);
-    const cudaError_t q = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, sample_tc_kernel<CHI, PER_SM>, tc::Cfg<CHI>::NT, smem);
-    if (q != cudaSuccess) cudaGetLastError();
-    if (raw_tiles == 2 || (q == cudaSuccess && fit >= PER_SM)) break;
-  }
   const int grid = sample_tc_grid(a.n_items, a.n_real, CHI, num_sms);
-  sample_tc_kernel<CHI, PER_SM><<<grid, tc::Cfg<CHI>::NT, smem, st>>>(a, raw_tiles);
+  sample_tc_kernel<CHI, PER_SM><<<grid, tc::Cfg<CHI>::NT, sample_tc_smem<CHI>(a.L), st>>>(a);
   return cudaGetLastError();
 }
 
