@@ -344,7 +344,9 @@ tnmc_status tnmc_env_build_occupancy(int L, int chi, int precision, int32_t* cta
                                      int32_t* num_sms);
 
 /* Device memory accounting.  tnmc_device_bytes: bytes the context holds now (its buffers
- * grow once to the largest n passed to tnmc_propose).  tnmc_estimate_device_bytes: bytes a
+ * grow once to the largest n passed to tnmc_propose; for chi <= 16 the first call for many
+ * proposals, of tnmc_propose or tnmc_eval_conditionals, adds workspace of the sampler, and goes
+ * without it, more slowly, if there is no memory left).  tnmc_estimate_device_bytes: bytes a
  * context of these arguments would hold after proposals of up to n_max per chain, without
  * allocating anything (0 for invalid arguments); it uses the current device's SM count, or
  * 152 when no device is present. */

@@ -48,8 +48,9 @@ struct tnmc_ctx {
   int8_t* hfield_buf = nullptr;   // the buffer behind hfield, allocated at the first tnmc_set_fields
   const int* chain_of = nullptr;  // chain index of each realization's draws (periodic driver), or nullptr
   // sampling
-  void* work = nullptr;
-  void* work_tc = nullptr;        // workspace of the tensor-core sampler (mixed TF32 path)
+  bool tc = false;                // served by the tensor-core sampler (mixed TF32 path)
+  void* work = nullptr;           // workspace of the sampler that serves the context
+  void* more = nullptr;           // what calls for many proposals take in addition, from the first of them on
   uint32_t* packed = nullptr;
   double* logq = nullptr;
   int32_t* energy = nullptr;
@@ -172,13 +173,21 @@ tnmc_status check_status(tnmc_ctx* c) {
 // capacity estimate so that the two cannot drift apart.
 struct CtxSizes {
   size_t J, beta, seeds, pvec, nlimit, env, kdim, dqr, lam, logz, rowbuf, Rstore, mscratch, stats, status, rstatus,
-      work, work_tc, clamps, have_state, cur_logq, cur_energy, cur_magnet, cur_spins, acc;
+      work, clamps, have_state, cur_logq, cur_energy, cur_magnet, cur_spins, acc;
   size_t total() const {
     return J + beta + seeds + pvec + nlimit + env + kdim + dqr + lam + logz + rowbuf + Rstore + mscratch + stats +
-           status + rstatus + work + work_tc + clamps + have_state + cur_logq + cur_energy + cur_magnet + cur_spins +
+           status + rstatus + work + clamps + have_state + cur_logq + cur_energy + cur_magnet + cur_spins +
            acc;
   }
 };
+
+bool uses_tc(int precision, int CHI) { return precision == TNMC_MIXED_TF32 && tnmc::sample_tc_supported(CHI); }
+
+// Workspace of the context's sampler, for calls of n_items proposals of each of n_real realizations.
+tnmc::SampleWork sampler_work(int L, int CHI, int precision, int num_sms, int n_items, int n_real) {
+  return uses_tc(precision, CHI) ? tnmc::sample_tc_work(L, CHI, num_sms, n_items, n_real)
+                                 : tnmc::sample_work(L, CHI, precision, num_sms, n_items, n_real);
+}
 
 CtxSizes ctx_sizes(int L, int n_real, int CHI, int precision, int n_chains, int num_sms) {
   CtxSizes z{};
@@ -199,10 +208,7 @@ CtxSizes ctx_sizes(int L, int n_real, int CHI, int precision, int n_chains, int 
   z.stats = 4 * sizeof(long long) * R;
   z.status = sizeof(unsigned);
   z.rstatus = sizeof(unsigned) * R;
-  // one workspace: that of the sampler which serves the context
-  const bool tc = precision == TNMC_MIXED_TF32 && tnmc::sample_tc_supported(CHI);
-  z.work = tc ? 0 : tnmc::sample_work_bytes(L, CHI, precision, num_sms);
-  z.work_tc = tc ? tnmc::sample_tc_work_bytes(L, CHI, num_sms) : 0;
+  z.work = sampler_work(L, CHI, precision, num_sms, 1, n_real).base;
   z.clamps = 8 * R;
   z.have_state = 4 * chains; z.cur_logq = 8 * chains; z.cur_energy = 4 * chains; z.cur_magnet = 4 * chains;
   z.cur_spins = 4 * chains * words;
@@ -229,6 +235,20 @@ tnmc_status ensure_props(tnmc_ctx* c, int n) {
   if ((s = dalloc(c, &c->cur_idx, items * sizeof(int)))) return s;
   c->cap_n = n;
   return TNMC_OK;
+}
+
+// The sampler's further workspace, at the first call of n_items proposals per realization that takes it.  The
+// call goes without (slower, the same results) where there is no memory for it, and while the stream is being
+// captured, since the block has to outlive the graph.  It is kept with the context: graphs hold its address.
+void ensure_more(tnmc_ctx* c, int n_items) {
+  if (c->more) return;
+  const tnmc::SampleWork w = sampler_work(c->L, c->CHI, c->precision, c->num_sms, n_items, c->n_real);
+  if (!w.takes_more) return;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) { cudaGetLastError(); return; }
+  if (cap != cudaStreamCaptureStatusNone) return;
+  const std::string err = c->err;
+  if (dalloc(c, &c->more, w.more) != TNMC_OK) c->err = err;
 }
 
 }  // namespace
@@ -289,6 +309,7 @@ tnmc_status tnmc_create(int L, int n_real, const int8_t* couplings, const double
   c->L = L; c->n_real = n_real; c->cap = n_real; c->chi = chi; c->CHI = round_chi(chi);
   c->precision = opts->precision; c->n_chains = opts->n_chains; c->n_therm = opts->n_therm;
   c->compression = opts->compression;
+  c->tc = uses_tc(c->precision, c->CHI);
   c->stream = reinterpret_cast<cudaStream_t>(opts->stream);
   c->words = (L * L + 31) / 32;
   cudaGetDevice(&c->device);
@@ -320,8 +341,7 @@ tnmc_status tnmc_create(int L, int n_real, const int8_t* couplings, const double
   TRY(dalloc(c, &c->stats, z.stats));
   TRY(dalloc(c, &c->status, z.status));
   TRY(dalloc(c, &c->rstatus, z.rstatus));
-  if (z.work) TRY(dalloc(c, &c->work, z.work));
-  if (z.work_tc) TRY(dalloc(c, &c->work_tc, z.work_tc));
+  TRY(dalloc(c, &c->work, z.work));
   TRY(dalloc(c, &c->clamps, z.clamps));
   const size_t chains = (size_t)n_real * c->n_chains;
   TRY(dalloc(c, &c->have_state, z.have_state));
@@ -468,19 +488,16 @@ static tnmc_status run_sample(tnmc_ctx* c, int n, uint64_t step0, const int8_t* 
   a.step0 = step0; a.J = c->J; a.beta = c->beta; a.seeds = c->seeds; a.env = c->env;
   a.spins_packed = props ? c->packed : nullptr; a.words = c->words;
   a.logq = logq; a.energy = props ? c->energy : nullptr; a.magnet = props ? c->magnet : nullptr;
-  a.clamps = props ? c->clamps : nullptr; a.forced = forced; a.qplus = qplus; a.work = c->work;
+  a.clamps = props ? c->clamps : nullptr; a.forced = forced; a.qplus = qplus;
   a.status = c->status;
   a.real_status = props ? c->rstatus : nullptr;
   a.hfield = c->hfield;
   a.chain_of = props ? c->chain_of : nullptr;
   a.kdim = c->kdim;
-  cudaError_t e;
-  if (c->work_tc) {
-    a.work = c->work_tc;
-    e = tnmc::launch_sample_tc(a, c->CHI, c->num_sms, c->stream);
-  } else {
-    e = tnmc::launch_sample(a, c->precision, c->CHI, c->num_sms, c->stream);
-  }
+  ensure_more(c, a.n_items);
+  a.work = c->work; a.more = c->more;
+  const cudaError_t e = c->tc ? tnmc::launch_sample_tc(a, c->CHI, c->num_sms, c->stream)
+                              : tnmc::launch_sample(a, c->precision, c->CHI, c->num_sms, c->stream);
   if (e != cudaSuccess) return cuda_fail(c, e, "sample launch");
   ++c->launches;
   return TNMC_OK;
@@ -733,8 +750,14 @@ size_t tnmc_estimate_device_bytes(int L, int n_real, int chi, const tnmc_opts* o
     cudaGetLastError();
     sms = 152;  // without a device: the GB300 count, for planning on a host
   }
-  return ctx_sizes(L, n_real, round_chi(chi), opts->precision, opts->n_chains, sms).total() +
-         (n_max > 0 ? props_bytes(L, n_real, opts->n_chains, n_max) : 0);
+  size_t b = ctx_sizes(L, n_real, round_chi(chi), opts->precision, opts->n_chains, sms).total();
+  if (n_max > 0) {
+    const int64_t items = (int64_t)opts->n_chains * n_max;
+    const tnmc::SampleWork w = sampler_work(L, round_chi(chi), opts->precision, sms,
+                                            (int)(items < (1 << 30) ? items : 1 << 30), n_real);
+    b += props_bytes(L, n_real, opts->n_chains, n_max) + (w.takes_more ? w.more : 0);
+  }
+  return b;
 }
 
 tnmc_status tnmc_copy_env(tnmc_ctx* c, int real, int row, double* tiles_host, int32_t* dims_host, double* lam_host) {

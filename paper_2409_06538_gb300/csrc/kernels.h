@@ -79,8 +79,11 @@ struct SampleArgs {
   // teacher forcing
   const int8_t* forced;            // [item][L*L] +-1 or nullptr (then Philox draws)
   double* qplus;                   // [item][L*L] (nullable)
-  // scratch
-  void* work;                      // [grid][warps][L][2*CHI] of compute type
+  // scratch, in slots of L x 2 CHI elements of the compute type for each of the proposals in flight: 32 of a
+  // warp (FMA samplers), 128 of a CTA (tensor-core sampler)
+  void* work;                      // the slots that every context has
+  void* more;                      // further ones that the build for many proposals takes (nullable: it does without)
+  int work_slots;                  // slots in work (set by the launch)
   unsigned* status;
   unsigned* real_status;           // [real] per-realization status bits (nullable)
   const int8_t* hfield;            // [real][L][L] external fields in units of beta (nullable)
@@ -94,8 +97,12 @@ bool sample_tc_supported(int CHI);
 // Self-test of the sampler's bounded mbarrier wait (see sample_tc.cu).
 cudaError_t launch_wait_probe(int arrive, long long limit, unsigned* status_dev, cudaStream_t st);
 cudaError_t launch_sample_tc(const SampleArgs& a, int CHI, int num_sms, cudaStream_t st);
-size_t sample_tc_work_bytes(int L, int CHI, int num_sms);
-size_t sample_work_bytes(int L, int CHI, int precision, int num_sms);
+
+// Workspace of the sampler that serves (precision, CHI): what every context holds, what a call for many
+// proposals takes in addition, and whether one for n_items of each of n_real realizations does.
+struct SampleWork { size_t base, more; bool takes_more; };
+SampleWork sample_work(int L, int CHI, int precision, int num_sms, int n_items, int n_real);
+SampleWork sample_tc_work(int L, int CHI, int num_sms, int n_items, int n_real);
 
 struct AcceptArgs {
   int L, n_real, n_chains, n, words, n_therm;

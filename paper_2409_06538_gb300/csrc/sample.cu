@@ -110,7 +110,8 @@ sample_thread_kernel(SampleArgs a, int n_slots) {
   const int tiles_per_real = (a.n_items + 31) / 32;
   const int64_t total = (int64_t)tiles_per_real * a.n_real;
   // v_y of every site of a row, [site][y][al][proposal]
-  T* work = reinterpret_cast<T*>(a.work) + (size_t)slot * L * 2 * CHI * 32 + lane;
+  const bool own = slot < a.work_slots;
+  T* work = reinterpret_cast<T*>(own ? a.work : a.more) + (size_t)(own ? slot : slot - a.work_slots) * L * 2 * CHI * 32 + lane;
 
   for (int64_t tile = slot; tile < total; tile += n_slots) {
     const int real = (int)(tile / tiles_per_real);
@@ -760,7 +761,8 @@ constexpr int kSampleWarps = 8;
 
 // Warps of sample_thread_kernel with a workspace of their own: kThreadWarps per SM, fewer where that
 // would take more than 256 MB, but never less than one per SM (32 proposals, as many as sample_kernel
-// has in flight).
+// has in flight).  One per SM is what every context has (a.work); the others are allocated at the first call
+// that this kernel serves with more, so that contexts of few proposals do not hold them.
 template <typename T>
 static int thread_slots(int L, int CHI, int num_sms) {
   const size_t per_warp = (size_t)L * 2 * CHI * 32 * sizeof(T), cap = (size_t)256 << 20;
@@ -769,15 +771,35 @@ static int thread_slots(int L, int CHI, int num_sms) {
   return (int)(slots < (size_t)num_sms ? (size_t)num_sms : slots);
 }
 
+// Whether one thread per proposal serves a call, with this many slots: from a number of proposals on; below
+// it, too few warps are in flight and one thread's chain over the bond index is what the call waits for.
+// Its time is the same for any number that the slots hold at once, that of the other kernel goes by the CTAs
+// (eight proposals of a realization each) that an SM gets.  propose() at L = 16, one GB300, ms of this kernel
+// (first) and of the other one at 1, 2 and 4 CTAs per SM:
+//   FP32 chi = 4  0.39 | 0.40 0.49 0.75     FP64 chi = 4   2.7 | 2.5 4.8  9.6
+//   FP32 chi = 8  0.67 | 0.42 0.49 0.79     FP64 chi = 8   4.9 | 2.7 5.2 13.0
+//   FP32 chi = 16 1.40 | 0.47 0.59 1.00     FP64 chi = 16 10.8 | 3.1 6.0 15.1
+// (BF16 as FP32; beyond 4 the other kernel's grow in proportion).  The line is drawn where this kernel is the
+// faster one in propose() and in eval_conditionals().  With more tiles than slots (large L, or without the
+// further slots) each further pass over the slots costs as much again.
+template <typename T>
+static bool takes_threads(int CHI, int num_sms, int n_items, int n_real, int64_t slots) {
+  if (CHI > 16) return false;
+  const int limit = sizeof(T) == 4 ? (CHI == 4 ? 1 : 4) : (CHI == 16 ? 3 : 1);
+  const int64_t ctas = (int64_t)((n_items + kSampleWarps - 1) / kSampleWarps) * n_real;
+  const int64_t tiles = (int64_t)((n_items + 31) / 32) * n_real, passes = (tiles + slots - 1) / slots;
+  return ctas > (passes > 1 ? 4 * passes : limit) * num_sms;
+}
+
 template <typename T, typename TE, int CHI>
-static cudaError_t launch_sample_thread(const SampleArgs& a, int num_sms, cudaStream_t st) {
+static cudaError_t launch_sample_thread(SampleArgs a, int64_t slots, int num_sms, cudaStream_t st) {
   const size_t smem = 4 * ((size_t)kThreadStages * 2 * CHI * CHI * sizeof(TE) + 2 * (size_t)((a.L + 15) & ~15) +
                            (size_t)((a.L + 31) / 32) * 128);
   cudaError_t e = allow_shared_memory<sample_thread_kernel<T, TE, CHI>>();
   if (e != cudaSuccess) return e;
   const int64_t tiles = (int64_t)((a.n_items + 31) / 32) * a.n_real;
-  int64_t slots = thread_slots<T>(a.L, CHI, num_sms);
   if (slots > tiles) slots = tiles;
+  a.work_slots = num_sms;
   sample_thread_kernel<T, TE, CHI><<<(unsigned)((slots + 3) / 4), 128, smem, st>>>(a, (int)slots);
   return cudaGetLastError();
 }
@@ -786,22 +808,8 @@ template <typename T, typename TE, int CHI>
 static cudaError_t launch_sample_t(const SampleArgs& a, int num_sms, cudaStream_t st) {
   constexpr int NW = kSampleWarps;
   if constexpr (CHI <= 16) {
-    // One thread per proposal from a number of proposals on; below it, too few warps are in flight and
-    // one thread's chain over the bond index is what the call waits for.  Its time is the same for any
-    // number that the slots hold at once, that of the other kernel goes by the CTAs (NW proposals of a
-    // realization each) that an SM gets.  propose() at L = 16, one GB300, ms of this kernel (first) and
-    // of the other one at 1, 2 and 4 CTAs per SM:
-    //   FP32 chi = 4  0.39 | 0.40 0.49 0.75     FP64 chi = 4   2.7 | 2.5 4.8  9.6
-    //   FP32 chi = 8  0.67 | 0.42 0.49 0.79     FP64 chi = 8   4.9 | 2.7 5.2 13.0
-    //   FP32 chi = 16 1.40 | 0.47 0.59 1.00     FP64 chi = 16 10.8 | 3.1 6.0 15.1
-    // (BF16 as FP32; beyond 4 the other kernel's grow in proportion).  The line is drawn where this
-    // kernel is the faster one in propose() and in eval_conditionals().  With more tiles than slots
-    // (large L) each further pass over the slots costs as much again.
-    constexpr int kLimit = sizeof(T) == 4 ? (CHI == 4 ? 1 : 4) : (CHI == 16 ? 3 : 1);
-    const int64_t ctas = (int64_t)((a.n_items + NW - 1) / NW) * a.n_real;
-    const int64_t tiles = (int64_t)((a.n_items + 31) / 32) * a.n_real, slots = thread_slots<T>(a.L, CHI, num_sms);
-    const int64_t passes = (tiles + slots - 1) / slots;
-    if (ctas > (passes > 1 ? 4 * passes : kLimit) * num_sms) return launch_sample_thread<T, TE, CHI>(a, num_sms, st);
+    const int64_t slots = a.more ? thread_slots<T>(a.L, CHI, num_sms) : num_sms;
+    if (takes_threads<T>(CHI, num_sms, a.n_items, a.n_real, slots)) return launch_sample_thread<T, TE, CHI>(a, slots, num_sms, st);
   }
   const size_t smem = sample_smem<CHI, NW>(a.L, sizeof(TE));
   constexpr auto kern = [] {
@@ -823,15 +831,19 @@ static cudaError_t launch_sample_t(const SampleArgs& a, int num_sms, cudaStream_
   return cudaGetLastError();
 }
 
-size_t sample_work_bytes(int L, int CHI, int precision, int num_sms) {
-  const size_t el = precision == 0 ? 8 : 4;
-  size_t b = (size_t)num_sms * 4 * kSampleWarps * (size_t)L * 2 * CHI * el;
+SampleWork sample_work(int L, int CHI, int precision, int num_sms, int n_items, int n_real) {
+  const size_t slot = (size_t)L * 2 * CHI * 32 * (precision == 0 ? 8 : 4);
+  static_assert(4 * kSampleWarps == 32, "sample_kernel has one slot of 32 proposals per SM");
+  SampleWork w{(size_t)num_sms * slot, 0, false};
   if (CHI <= 16) {
-    const size_t slots = precision == 0 ? thread_slots<double>(L, CHI, num_sms) : thread_slots<float>(L, CHI, num_sms);
-    const size_t t = slots * (size_t)L * 2 * CHI * 32 * el;
-    if (t > b) b = t;
+    const int slots = precision == 0 ? thread_slots<double>(L, CHI, num_sms) : thread_slots<float>(L, CHI, num_sms);
+    const int64_t tiles = (int64_t)((n_items + 31) / 32) * n_real;
+    w.more = (size_t)(slots - num_sms) * slot;
+    w.takes_more = w.more > 0 && tiles > num_sms &&
+                   (precision == 0 ? takes_threads<double>(CHI, num_sms, n_items, n_real, slots)
+                                   : takes_threads<float>(CHI, num_sms, n_items, n_real, slots));
   }
-  return b;
+  return w;
 }
 
 cudaError_t launch_sample(const SampleArgs& a, int precision, int CHI, int num_sms, cudaStream_t st) {

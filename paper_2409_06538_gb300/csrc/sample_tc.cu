@@ -376,7 +376,9 @@ __global__ void __launch_bounds__(tc::Cfg<CHI>::NT, PER_SM) sample_tc_kernel(Sam
     };
     // R_{c+1}(y) per site and proposal, [site][y][j / 4][proposal][4]: 16-byte accesses that are
     // contiguous over the lanes
-    float* work = reinterpret_cast<float*>(a.work) + (size_t)blockIdx.x * L * 2 * M * CHI + 4 * tid;
+    const bool own = (int)blockIdx.x < a.work_slots;
+    float* work = reinterpret_cast<float*>(own ? a.work : a.more) +
+                  (size_t)(own ? (int)blockIdx.x : (int)blockIdx.x - a.work_slots) * L * 2 * M * CHI + 4 * tid;
     float* rws = Rws + 4 * tid;                       // one site's, in shared memory
 
     for (int64_t tileid = blockIdx.x; run && tileid < total; tileid += gridDim.x) {
@@ -633,29 +635,32 @@ static size_t sample_tc_smem(int L) {
          (size_t)8 * ((L + 15) & ~15) + (size_t)words_row * tc::M * sizeof(uint32_t) + 64;
 }
 
-static int per_sm(int CHI) { return CHI <= 16 ? tc::Cfg<16>::PER_SM : tc::Cfg<32>::PER_SM; }
+static int64_t sample_tc_tiles(int n_items, int n_real) { return (int64_t)((n_items + tc::M - 1) / tc::M) * n_real; }
 
-static int sample_tc_grid(int n_items, int n_real, int CHI, int num_sms) {
-  const int64_t tiles = (int64_t)((n_items + tc::M - 1) / tc::M) * n_real;
-  int64_t grid = (int64_t)num_sms * per_sm(CHI);
-  if (grid > tiles) grid = tiles;
-  return grid < 1 ? 1 : (int)grid;
-}
+// Every context has the slots of two CTAs per SM; those of the third at CHI = 16 are allocated at the first call
+// whose tiles two do not hold at once.
+constexpr int kOwnSlots = 2;
 
-size_t sample_tc_work_bytes(int L, int CHI, int num_sms) {
-  return (size_t)num_sms * per_sm(CHI) * (size_t)L * 2 * tc::M * CHI * sizeof(float);
+SampleWork sample_tc_work(int L, int CHI, int num_sms, int n_items, int n_real) {
+  const size_t slot = (size_t)L * 2 * tc::M * CHI * sizeof(float);
+  const int per_sm = CHI <= 16 ? tc::Cfg<16>::PER_SM : tc::Cfg<32>::PER_SM;
+  return SampleWork{kOwnSlots * num_sms * slot, (per_sm - kOwnSlots) * num_sms * slot,
+                    per_sm > kOwnSlots && sample_tc_tiles(n_items, n_real) > (int64_t)kOwnSlots * num_sms};
 }
 
 template <int CHI, int PER_SM>
-static cudaError_t launch_tc_t(const SampleArgs& a, int num_sms, cudaStream_t st) {
-  // Where two CTAs per SM hold every tile anyway, the build with their registers (CHI = 16: 48 tiles
-  // 2.8 -> 2.6 ms, while 16384 tiles take 158 ms with two CTAs per SM against 140 with three).
-  if constexpr (PER_SM > 2)
-    if (sample_tc_grid(a.n_items, a.n_real, CHI, num_sms) <= 2 * num_sms) return launch_tc_t<CHI, 2>(a, num_sms, st);
+static cudaError_t launch_tc_t(SampleArgs a, int num_sms, cudaStream_t st) {
+  const int64_t tiles = sample_tc_tiles(a.n_items, a.n_real);
+  // Where two CTAs per SM hold every tile anyway, or there is no workspace for a third, the build with their
+  // registers (CHI = 16: 48 tiles 2.8 -> 2.6 ms, while 16384 tiles take 158 ms with two CTAs per SM against
+  // 140 with three).
+  if constexpr (PER_SM > kOwnSlots)
+    if (tiles <= (int64_t)kOwnSlots * num_sms || !a.more) return launch_tc_t<CHI, kOwnSlots>(a, num_sms, st);
   const cudaError_t e = allow_shared_memory<sample_tc_kernel<CHI, PER_SM>>();
   if (e != cudaSuccess) return e;
-  const int grid = sample_tc_grid(a.n_items, a.n_real, CHI, num_sms);
-  sample_tc_kernel<CHI, PER_SM><<<grid, tc::Cfg<CHI>::NT, sample_tc_smem<CHI>(a.L), st>>>(a);
+  a.work_slots = kOwnSlots * num_sms;
+  const int64_t most = (int64_t)num_sms * PER_SM, grid = tiles < most ? tiles : most;
+  sample_tc_kernel<CHI, PER_SM><<<(unsigned)grid, tc::Cfg<CHI>::NT, sample_tc_smem<CHI>(a.L), st>>>(a);
   return cudaGetLastError();
 }
 
