@@ -2,8 +2,8 @@
 // Sec. II.B reverse-order sampling, Figs. fig:Z4 / fig:ZS4), and the same sweep with given
 // spins (teacher forcing) for q(s) of arbitrary configurations.
 //
-// Two mappings with the same arithmetic, operation by operation, so that the choice between them
-// changes no result.  sample_thread_kernel (CHI <= 16): one thread per proposal, the whole bond index
+// Two mappings with the same arithmetic, operation by operation (which product of a sum is rounded before
+// it enters a fused multiply-add is written out in both), so that the choice between them changes no result.  sample_thread_kernel (CHI <= 16): one thread per proposal, the whole bond index
 // in its registers, a warp's 32 proposals sharing the environment tile in shared memory.
 // sample_kernel: one warp per proposal, lanes over the bond index; the CTA's warps are NW proposals of
 // the same realization and share every environment tile, staged once per site into shared memory
@@ -405,8 +405,8 @@ sample_kernel(SampleArgs a) {
           const int be = (al + t) & (CHI - 1);
           const T r0 = __shfl_sync(0xffffffffu, R0, be);
           const T r1 = __shfl_sync(0xffffffffu, R1, be);
-          v0 += env_load<T, TE>(tl[al * CHI + be]) * r0;
-          v1 += env_load<T, TE>(tl[CHI * CHI + al * CHI + be]) * r1;
+          v0 = tfma(env_load<T, TE>(tl[al * CHI + be]), r0, v0);
+          v1 = tfma(env_load<T, TE>(tl[CHI * CHI + al * CHI + be]), r1, v1);
         }
         if (!active_lane) { v0 = 0; v1 = 0; }
         if (active_lane) { work[(size_t)c * 2 * CHI + al] = v0; work[(size_t)c * 2 * CHI + CHI + al] = v1; }
@@ -417,8 +417,8 @@ sample_kernel(SampleArgs a) {
           if (r > 0) { const int sg = jv_s[c] * prow[c]; f0 = sg > 0 ? eb : ebm; f1 = sg > 0 ? ebm : eb; }
           if (hf) { const int kh = hf[(size_t)r * L + c]; if (kh) { f0 *= num<T>::exp_((T)(betad * kh)); f1 *= num<T>::exp_((T)(-betad * kh)); } }
           const T same = jh > 0 ? eb : ebm, diff = jh > 0 ? ebm : eb;
-          const T n0 = same * f0 * v0 + diff * f1 * v1;   // y' = +1
-          const T n1 = diff * f0 * v0 + same * f1 * v1;   // y' = -1
+          const T n0 = tfma(same * f0, v0, tmul(diff * f1, v1));   // y' = +1
+          const T n1 = tfma(diff * f0, v0, tmul(same * f1, v1));   // y' = -1
           T mx = tabs(n0) > tabs(n1) ? tabs(n0) : tabs(n1);
           mx = warp_max(mx);
           const T inv = mx > T(0) ? T(1) / mx : T(1);
@@ -446,7 +446,7 @@ sample_kernel(SampleArgs a) {
         }
         const T v0 = active_lane ? work[(size_t)c * 2 * CHI + al] : T(0);
         const T v1 = active_lane ? work[(size_t)c * 2 * CHI + CHI + al] : T(0);
-        T d0 = warp_sum(ell * v0), d1 = warp_sum(ell * v1);
+        T d0 = warp_sum(tmul(ell, v0)), d1 = warp_sum(tmul(ell, v1));
         T f0 = 1, f1 = 1;
         if (r > 0) { const int sg = jv_s[c] * prow[c]; f0 = sg > 0 ? eb : ebm; f1 = sg > 0 ? ebm : eb; }
         if (c > 0) { const int sg = jh_s[c - 1] * sprev; f0 *= sg > 0 ? eb : ebm; f1 *= sg > 0 ? ebm : eb; }
@@ -490,7 +490,7 @@ sample_kernel(SampleArgs a) {
 #pragma unroll 8
         for (int t = 0; t < CHI; ++t) {
           const T lt = __shfl_sync(0xffffffffu, ell, t);
-          acc += lt * env_load<T, TE>(bs[t * CHI + al]);
+          acc = tfma(lt, env_load<T, TE>(bs[t * CHI + al]), acc);
         }
         if (!active_lane) acc = 0;
         T mx = warp_max(tabs(acc));
