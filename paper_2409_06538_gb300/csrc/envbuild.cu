@@ -109,12 +109,6 @@ __device__ __forceinline__ void rotation_from_gram(float a, float b, float g, fl
   s = (d < 0.0f ? -g : g) * rinv * ic;
 }
 
-template <typename T> __device__ __forceinline__ T group8_sum(T v) {
-  v += __shfl_xor_sync(0xffffffffu, v, 1);
-  v += __shfl_xor_sync(0xffffffffu, v, 2);
-  v += __shfl_xor_sync(0xffffffffu, v, 4);
-  return v;
-}
 template <int ID> __device__ __forceinline__ void named_barrier(int nthreads) {
   asm volatile("bar.sync %0, %1;\n" ::"n"(ID), "r"(nthreads) : "memory");
 }
