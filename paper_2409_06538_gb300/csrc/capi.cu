@@ -755,7 +755,7 @@ size_t tnmc_estimate_device_bytes(int L, int n_real, int chi, const tnmc_opts* o
     const int64_t items = (int64_t)opts->n_chains * n_max;
     const tnmc::SampleWork w = sampler_work(L, round_chi(chi), opts->precision, sms,
                                             (int)(items < (1 << 30) ? items : 1 << 30), n_real);
-    b += props_bytes(L, n_real, opts->n_chains, n_max) + (w.takes_more ? w.more : 0);
+    b += props_bytes(L, n_real, opts->n_chains, n_max) + (w.up_to ? w.more : 0);
   }
   return b;
 }

@@ -99,8 +99,9 @@ cudaError_t launch_wait_probe(int arrive, long long limit, unsigned* status_dev,
 cudaError_t launch_sample_tc(const SampleArgs& a, int CHI, int num_sms, cudaStream_t st);
 
 // Workspace of the sampler that serves (precision, CHI): what every context holds, what a call for many
-// proposals takes in addition, and whether one for n_items of each of n_real realizations does.
-struct SampleWork { size_t base, more; bool takes_more; };
+// proposals takes in addition, and whether one for n_items of each of n_real realizations does, or one for at
+// most that many may (the rule is not monotone: a call that needs several passes over the slots can go without).
+struct SampleWork { size_t base, more; bool takes_more, up_to; };
 SampleWork sample_work(int L, int CHI, int precision, int num_sms, int n_items, int n_real);
 SampleWork sample_tc_work(int L, int CHI, int num_sms, int n_items, int n_real);
 

@@ -834,14 +834,18 @@ static cudaError_t launch_sample_t(const SampleArgs& a, int num_sms, cudaStream_
 SampleWork sample_work(int L, int CHI, int precision, int num_sms, int n_items, int n_real) {
   const size_t slot = (size_t)L * 2 * CHI * 32 * (precision == 0 ? 8 : 4);
   static_assert(4 * kSampleWarps == 32, "sample_kernel has one slot of 32 proposals per SM");
-  SampleWork w{(size_t)num_sms * slot, 0, false};
+  SampleWork w{(size_t)num_sms * slot, 0, false, false};
   if (CHI <= 16) {
     const int slots = precision == 0 ? thread_slots<double>(L, CHI, num_sms) : thread_slots<float>(L, CHI, num_sms);
     const int64_t tiles = (int64_t)((n_items + 31) / 32) * n_real;
     w.more = (size_t)(slots - num_sms) * slot;
-    w.takes_more = w.more > 0 && tiles > num_sms &&
-                   (precision == 0 ? takes_threads<double>(CHI, num_sms, n_items, n_real, slots)
-                                   : takes_threads<float>(CHI, num_sms, n_items, n_real, slots));
+    auto takes = [&](int64_t n_slots) {
+      return w.more > 0 && tiles > num_sms &&
+             (precision == 0 ? takes_threads<double>(CHI, num_sms, n_items, n_real, n_slots)
+                             : takes_threads<float>(CHI, num_sms, n_items, n_real, n_slots));
+    };
+    w.takes_more = takes(slots);
+    w.up_to = takes(tiles);               // as if one pass held them, which it does for some smaller call
   }
   return w;
 }

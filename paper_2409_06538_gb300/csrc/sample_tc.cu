@@ -644,8 +644,8 @@ constexpr int kOwnSlots = 2;
 SampleWork sample_tc_work(int L, int CHI, int num_sms, int n_items, int n_real) {
   const size_t slot = (size_t)L * 2 * tc::M * CHI * sizeof(float);
   const int per_sm = CHI <= 16 ? tc::Cfg<16>::PER_SM : tc::Cfg<32>::PER_SM;
-  return SampleWork{kOwnSlots * num_sms * slot, (per_sm - kOwnSlots) * num_sms * slot,
-                    per_sm > kOwnSlots && sample_tc_tiles(n_items, n_real) > (int64_t)kOwnSlots * num_sms};
+  const bool more = per_sm > kOwnSlots && sample_tc_tiles(n_items, n_real) > (int64_t)kOwnSlots * num_sms;
+  return SampleWork{kOwnSlots * num_sms * slot, (per_sm - kOwnSlots) * num_sms * slot, more, more};
 }
 
 template <int CHI, int PER_SM>
