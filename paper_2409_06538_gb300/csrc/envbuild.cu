@@ -80,35 +80,6 @@ __device__ __forceinline__ void rot16(double2& u, double2& v, double c, double s
   u = make_double2(rot_u(a.x, b.x, c, s), rot_u(a.y, b.y, c, s));
   v = make_double2(rot_v(a.x, b.x, c, s), rot_v(a.y, b.y, c, s));
 }
-// Jacobi rotation (c, s) that makes columns p, q orthogonal, from a = |y_p|^2, b = |y_q|^2,
-// g = y_p . y_q (y_p' = c y_p - s y_q, y_q' = s y_p + c y_q).  The angle solves
-// tan 2theta = 2g / (b - a) with |theta| <= pi/4:
-//   r = sqrt((b-a)^2 + 4 g^2), cos 2theta = |b-a| / r, c = sqrt((1 + cos 2theta) / 2),
-//   s = sgn(b-a) g / (r c)   (sgn(0) = +1),
-// two reciprocal square roots in sequence instead of the divide/sqrt chain of the tangent
-// form.  FP32 uses the hardware rsqrt with one Newton step each, so c^2 + s^2 = 1 to
-// working precision; FP64 calls the library's, which leaves out a root and a division each.
-__device__ __forceinline__ float rsqrt_nr(float x) {
-  const float r = rsqrtf(x);
-  return r * fmaf(-0.5f * x * r, r, 1.5f);
-}
-__device__ __forceinline__ void rotation_from_gram(double a, double b, double g, double& c, double& s) {
-  const double d = b - a;
-  const double rinv = rsqrt(fma(d, d, 4.0 * g * g));
-  const double h = fma(0.5 * fabs(d), rinv, 0.5);
-  const double ic = rsqrt(h);
-  c = h * ic;
-  s = (d < 0.0 ? -g : g) * rinv * ic;
-}
-__device__ __forceinline__ void rotation_from_gram(float a, float b, float g, float& c, float& s) {
-  const float d = b - a;
-  const float rinv = rsqrt_nr(fmaf(d, d, 4.0f * g * g));
-  const float h = fmaf(0.5f * fabsf(d), rinv, 0.5f);
-  const float ic = rsqrt_nr(h);
-  c = h * ic;
-  s = (d < 0.0f ? -g : g) * rinv * ic;
-}
-
 template <int ID> __device__ __forceinline__ void named_barrier(int nthreads) {
   asm volatile("bar.sync %0, %1;\n" ::"n"(ID), "r"(nthreads) : "memory");
 }
@@ -342,15 +313,6 @@ __device__ __forceinline__ double entry_max(double m, double) { return m; }
 // What an entry makes of its matrix: 0, 1 beyond kLargeEntry, 2 beyond what kDown brings back.
 template <typename T> __device__ __forceinline__ void note_large(T entry, int* flag) {
   if (kLate<T> && entry > T(kLargeEntry)) atomicMax(flag, entry * T(kDown) > T(kLargeEntry) ? 2 : 1);
-}
-
-// Square root of a column's squared norm.  In FP64 from the reciprocal root and one step of Newton's
-// iteration, s + (ss - s^2) / (2 s): half the instructions of the pipe that the factorisation waits for.
-__device__ __forceinline__ float norm_of(float ss) { return sqrtf(ss); }
-__device__ __forceinline__ double norm_of(double ss) {
-  if (!(ss > 0.0 && ss < INFINITY)) return ss;
-  const double r = rsqrt(ss), s = ss * r;
-  return fma(0.5 * r, fma(-s, s, ss), s);
 }
 
 // Reflector of column j, by the warp that owns it; j lies in the rows of run C0.
