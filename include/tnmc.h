@@ -338,8 +338,11 @@ tnmc_status tnmc_selftest_bounded_wait(int arrive, int64_t* elapsed_us);
  * realizations (one CTA each) one SM holds at once for this L, chi and precision (shared
  * memory and registers decide), *num_sms (nullable) the SM count.  A batch of R
  * realizations fills R of ctas_per_sm * num_sms slots; callers size the number of batches
- * they keep in flight from it.  TNMC_ERR_ARG / TNMC_ERR_UNSUPPORTED for bad arguments,
- * TNMC_ERR_CUDA without a device. */
+ * they keep in flight from it.  For chi in 9..16 outside FP64 there is a second build of the kernel,
+ * seven realizations per SM at about 4/3 of the time a wave; a call whose own R saves waves by
+ * it uses it (same results), never one of R <= ctas_per_sm * num_sms.  The count given is the
+ * first build's, which batches in flight side by side go through.  TNMC_ERR_ARG /
+ * TNMC_ERR_UNSUPPORTED for bad arguments, TNMC_ERR_CUDA without a device. */
 tnmc_status tnmc_env_build_occupancy(int L, int chi, int precision, int32_t* ctas_per_sm,
                                      int32_t* num_sms);
 

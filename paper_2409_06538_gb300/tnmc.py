@@ -48,7 +48,8 @@ def nishimori_beta(p):
 
 
 def env_build_occupancy(L, chi, precision="tf32"):
-    """(realizations per SM, SM count) for the environment build on the current device."""
+    """(realizations per SM, SM count) for the environment build on the current device (for chi 9..16 of the
+    build that serves batches of up to their product; larger ones may take another with seven per SM)."""
     lib = _capi.load()
     per, sms = _c.c_int32(0), _c.c_int32(0)
     _capi.check(lib.tnmc_env_build_occupancy(int(L), int(chi), _capi.PRECISIONS[precision], _c.byref(per),
