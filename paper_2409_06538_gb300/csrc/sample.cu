@@ -3,8 +3,9 @@
 // spins (teacher forcing) for q(s) of arbitrary configurations.
 //
 // Two mappings with the same arithmetic, operation by operation (which product of a sum is rounded before
-// it enters a fused multiply-add is written out in both), so that the choice between them changes no result.  sample_thread_kernel (CHI <= 16): one thread per proposal, the whole bond index
-// in its registers, a warp's 32 proposals sharing the environment tile in shared memory.
+// it enters a fused multiply-add is written out in both), so that the choice between them changes no
+// result.  sample_thread_kernel (CHI <= 16): one thread per proposal, the whole bond index in its
+// registers, a warp's 32 proposals sharing the environment tile in shared memory.
 // sample_kernel: one warp per proposal, lanes over the bond index; the CTA's warps are NW proposals of
 // the same realization and share every environment tile, staged once per site into shared memory
 // with cp.async double buffering.  For row r (fields h_c = beta Jv[r-1][c] s_{r-1,c}):
