@@ -480,6 +480,7 @@ __global__ void __launch_bounds__(tc::Cfg<CHI>::NT, PER_SM) sample_tc_kernel(Sam
 
         __threadfence();              // the copies below read what this thread has stored
         // ---------------- left sweep ----------------
+        tmem_wait_st();               // stores are in no order of their own: R_1's before those of l
         put_e0<CHI>(ta);
         a_ready();
         int sprev = 0;
