@@ -834,7 +834,9 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
       const T tinyY = sumY * num<T>::eps * num<T>::eps;
       if (zip) {
         // the zip-up's Y = M is graded by columns (P = U S), where the one-sided Jacobi is
-        // accurate without preconditioning
+        // accurate without preconditioning; it is not near to orthogonal, though: in the first four
+        // sweeps nearly all pairs above the threshold rotate (8 to 10 sweeps a site at chi = 32,
+        // 3.4 to 4 on the preconditioned matrix)
         for (int e = tid; e < DP * npad; e += NT) { const int i = e % DP, j = e / DP; Vc[e] = (i == j) ? T(1) : T(0); }
         for (int e = tid; e < DP * (npad - n); e += NT) Yc[(size_t)n * DP + e] = T(0);
         __syncthreads();
@@ -1021,10 +1023,11 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
                 get(col(Yc, pa), ya);
                 int t0 = 0;
                 // The test pays where few block pairs rotate: on the preconditioned matrix in FP32
-                // at once, on the zip-up's M (a third of the block pairs in the first sweep, an
-                // eighth in the fifth) from the sixth sweep on (L = 48, chi = 32: 277 ms, from the
-                // third 288, never 288), in FP64, whose tolerance asks for more rotations, from the
-                // third on.
+                // at once, on the zip-up's M (of the live block pairs 74, 54, 48, 42, 34, 24, 15 and
+                // 9 % rotate in the sweeps of a chi = 32 site at L = 48; 66 to 24 % in the first five
+                // at L = 24, 77 to 38 % at L = 64, 48 to 14 % at chi = 64) from the sixth sweep on
+                // (L = 48, chi = 32: 277 ms, from the third 288, never 288), in FP64, whose tolerance
+                // asks for more rotations, from the third on.
                 if (sizeof(T) == 8 ? sweep >= 2 : (!zip || sweep >= 5)) {
                   T v[9];               // A's norm, four products, the four norms of block B
                   v[0] = norm_a(ya);
