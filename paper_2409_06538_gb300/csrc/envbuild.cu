@@ -298,21 +298,27 @@ template <typename T> struct QrOut {
 // where a division occupies the FP64 pipe, only the pivot's warp does.
 template <typename T> constexpr bool kLate = sizeof(T) == 4;
 
-// The range of inverse() ends at a coefficient of 8e37, at most twice a column's squared norm.  A matrix that
-// may go beyond it (weights of exp(36) and more: strong fields, low temperatures) is factored times kDown, a
-// power of two, so nothing is rounded by it; nothing has to be scaled back either, as R is normalised, the
-// right singular vectors have no scale and the singular values are only compared.  One that is too large for
-// that as well becomes NaN, which the sampler flags.  Whoever forms a matrix looks at its entries, and the
-// scaling is out of line: that costs 1 % of the builds for chi <= 8, 4 % of the crowd's, whose code is the
-// tightest (90.5 -> 93.9 ms, 1024 realizations of 32 x 32), and nothing beyond.  A test of each coefficient in
-// the warps that use it cost 2 to 4 % of all, in the pivot's warp 3 to 8 %, a second body that divides 1 to 3 %.
-constexpr float kLargeEntry = 1e16f;                 // 2 * 128 * 128 entries * kLargeEntry^2 = 3.3e36
-constexpr float kDown = 1.0f / 4294967296.0f;        // 2^-32
+// Ranges of the FP32 build.  inverse() ends at a coefficient of 8e37, at most twice a column's squared norm;
+// the Jacobi multiplies two squared norms.  A matrix with an entry beyond the limits below (weights of exp(16)
+// and more: strong fields, low temperatures) is factored times a power of two that brings its largest entry
+// just below the limit, so nothing is rounded by it; nothing has to be scaled back either, as R is normalised,
+// the right singular vectors have no scale and the singular values are only compared.  One that has overflowed
+// becomes NaN, which the sampler flags.  Whoever forms a matrix looks at its entries, and the scaling is out of
+// line: that costs 1 % of the builds for chi <= 8, 4 % of the crowd's, whose code is the tightest (90.5 -> 93.9
+// ms, 1024 realizations of 32 x 32), and nothing beyond.  A test of each coefficient in the warps that use it
+// cost 2 to 4 % of all, in the pivot's warp 3 to 8 %, a second body that divides 1 to 3 %.
+constexpr float kLargeX = 1125899906842624.0f;       // 2^50: 2 * 256 entries * kLargeX^2 = 6.5e32
+constexpr float kLargeY = 8388608.0f;                // 2^23: (128 * 128 entries * kLargeY^2)^2 = 1.3e36
 __device__ __forceinline__ float entry_max(float m, float x) { return fmaxf(m, fabsf(x)); }
 __device__ __forceinline__ double entry_max(double m, double) { return m; }
-// What an entry makes of its matrix: 0, 1 beyond kLargeEntry, 2 beyond what kDown brings back.
-template <typename T> __device__ __forceinline__ void note_large(T entry, int* flag) {
-  if (kLate<T> && entry > T(kLargeEntry)) atomicMax(flag, entry * T(kDown) > T(kLargeEntry) ? 2 : 1);
+// Leaves the bits of the largest entry beyond the limit in flag (0: none).
+template <typename T> __device__ __forceinline__ void note_large(T entry, float limit, int* flag) {
+  if (kLate<T> && entry > T(limit)) atomicMax(flag, __float_as_int((float)entry));
+}
+// The power of two that takes such an entry into [limit / 2, limit), NaN for an infinity.
+__device__ __forceinline__ float down_scale(float limit, int bits) {
+  const int e = bits >> 23, to = (__float_as_int(limit) >> 23) - 1;
+  return e == 255 ? NAN : __int_as_float((127 + to - e) << 23);
 }
 
 // Reflector of column j, by the warp that owns it; j lies in the rows of run C0.
@@ -601,11 +607,10 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
           }
         }
       }
-      note_large(xmax, &large_s);
+      note_large(xmax, kLargeX, &large_s);
       __syncthreads();
       if (kLate<T> && large_s) {
-        const T s = large_s > 1 ? T(NAN) : T(kDown);
-        scale_matrix<T>(Xs, 2 * D, D, 2 * D, s, tid, NT);
+        scale_matrix<T>(Xs, 2 * D, D, 2 * D, T(down_scale(kLargeX, large_s)), tid, NT);
         __syncthreads();
       }
       // the next site's tile streams in while the QR runs
@@ -763,19 +768,19 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
       // prefetched): 4 x 4 register tiles over (rows, compact columns).  Zip-up: Y = M (the
       // previous row is canonical on the side not yet swept, so no R factor)
       constexpr int VK = C::VT / NT;
-      T fro[VK] = {};
+      T fro[VK] = {}, ymax = 0;
       if (zip) {
         for (int e = tid; e < DP * n; e += NT) {
           const int i = e % DP, j = e / DP;
           const T v = i < D ? Mc[(size_t)j * D + i] : T(0);
           Yc[e] = v;
+          ymax = entry_max(ymax, v);
 #pragma unroll
           for (int q = 0; q < VK; ++q) if ((e / NT) % VK == q) fro[q] += v * v;
         }
       } else {
         constexpr int TI = D / 4;
         const int TJ = (n + 3) / 4;
-        T ymax = 0;
         for (int u = tid; u < TI * TJ; u += NT) {
           const int i0 = (u % TI) * 4, j0 = (u / TI) * 4;
           T acc[4][4] = {};
@@ -809,8 +814,8 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
             }
           }
         }
-        note_large(ymax, &large_s);
       }
+      note_large(ymax, kLargeY, &large_s);
       // the Jacobi runs on npad = n rounded up to 8 columns (blocks of 4, an even number of
       // blocks); columns n..npad-1 of Y are zero and never rotate
       const int npad = (n + 7) & ~7;
@@ -822,9 +827,8 @@ env_build_kernel(EnvBuildArgs<T, TE> args) {
       if (tid == 0) { rot[0] = 0; rot[1] = 0; rot[2] = 0; }
       __syncthreads();
       T sumY = warp_sum(lane < C::VT / 32 ? red[lane] : T(0));
-      if (kLate<T> && large_s) {             // (never set in zip-up mode)
-        const T s = large_s > 1 ? T(NAN) : T(kDown);
-        T f = scale_matrix<T>(Yc, D, n, DP, s, tid, NT);
+      if (kLate<T> && large_s) {
+        T f = scale_matrix<T>(Yc, D, n, DP, T(down_scale(kLargeY, large_s)), tid, NT);
         f = warp_sum(f);
         __syncthreads();
         if (lane == 0) red[warp] = f;
